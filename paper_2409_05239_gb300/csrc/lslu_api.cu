@@ -147,6 +147,11 @@ lslu_status create_common(lslu_ctx* c, const int64_t* rp, const int32_t* ci, con
   CKC(cudaMemset(c->D, 0, (size_t)c->ldd * (K + 1) * bb));
   CKC(dmalloc(&c->H, (size_t)P * c->h_stride));
   CKC(dmalloc(&c->W, (size_t)P * c->w_stride));
+  // a solve writes the upper Hessenberg part of H (triangle of W) only, and
+  // the projected solve and lslu_get_state read whole columns: what cudaMalloc
+  // left below must be zero
+  CKC(cudaMemset(c->H, 0, (size_t)P * c->h_stride * sizeof(double)));
+  CKC(cudaMemset(c->W, 0, (size_t)P * c->w_stride * sizeof(double)));
   CKC(cudaMalloc(&c->TLi, (size_t)P * c->t_stride * bb));
   CKC(cudaMalloc(&c->TDi, (size_t)P * c->t_stride * bb));
   CKC(dmalloc(&c->gp, (size_t)P * K));
