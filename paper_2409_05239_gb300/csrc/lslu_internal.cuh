@@ -94,7 +94,13 @@ struct DevCsr {
   int compressed = 0;          // 16-bit column offsets available (off, ubase)
   int use_cmp = 0;             // the shape reads them (shape >= kShapesPerFormat)
   uint16_t* off = nullptr;     // nnz_padded: column - first column of its 8-entry unit
-  int32_t* ubase = nullptr;    // nnz_padded / 8: first column of every unit
+  int32_t* ubase = nullptr;    // nnz_padded / 8: smallest column of every unit (of its block
+                               // with block_compressed)
+  int block_compressed = 0;    // every kPermBlock-entry block spans < 2^16 columns: offsets
+                               // count from the block's smallest column
+  int32_t* bbase = nullptr;    // smallest column of every block, row by row
+  int32_t* rblk = nullptr;     // rows: first block of every row
+  int num_sms = 0;             // of the device it lives on
   int64_t rows = 0, cols = 0;
   int64_t nnz = 0;         // true non-zeros
   int64_t nnz_padded = 0;  // entries stored, including padding

@@ -30,11 +30,23 @@ constexpr int kRowsPerBlock = 256 / kGroup;
 // the single-vector product of the default 16-lane shapes bit for bit (16x2 on
 // 32-bit columns, 16x1 on 16-bit offsets).
 
-// Columns of the lane's next chunk (C entries at position p of the row
-// storage): 32-bit indices (C = 4) or a unit of 16-bit offsets (C = 8).
-template <bool CMP>
-__device__ __forceinline__ void chunk_cols(const ColIdx& ci, int32_t p, int32_t (&c)[CMP ? 8 : 4]) {
-  if constexpr (CMP) {
+template <int F>
+constexpr int kFmtChunk = F == kFmtUnit8 ? 8 : 4;
+
+// Columns of the lane's next chunk (entry e of the row, at position p of the
+// storage): 8 entries in kFmtUnit8, else 4.
+template <int F>
+__device__ __forceinline__ void chunk_cols(const ColIdx& ci, int32_t p, int32_t e, int32_t blk,
+                                           int32_t (&c)[kFmtChunk<F>]) {
+  if constexpr (F == kFmtUnit4 || F == kFmtBlock4) {
+    const uint2 o = ld_stream_off4(ci.off + p);
+    const int32_t b =
+        F == kFmtBlock4 ? __ldg(ci.bbase + blk + e / kPermBlock) : __ldg(ci.ubase + (p >> 3));
+    c[0] = b + (int32_t)(o.x & 0xffffu);
+    c[1] = b + (int32_t)(o.x >> 16);
+    c[2] = b + (int32_t)(o.y & 0xffffu);
+    c[3] = b + (int32_t)(o.y >> 16);
+  } else if constexpr (F == kFmtUnit8) {
     const uint4 o = ld_stream_off(ci.off + p);
     const int32_t b = __ldg(ci.ubase + (p >> 3));
     const uint32_t w[4] = {o.x, o.y, o.z, o.w};
@@ -49,9 +61,9 @@ __device__ __forceinline__ void chunk_cols(const ColIdx& ci, int32_t p, int32_t 
   }
 }
 
-template <typename VT, bool CMP>
-__device__ __forceinline__ void chunk_vals(const VT* val, int32_t p, float (&v)[CMP ? 8 : 4]) {
-  if constexpr (CMP)
+template <typename VT, int F>
+__device__ __forceinline__ void chunk_vals(const VT* val, int32_t p, float (&v)[kFmtChunk<F>]) {
+  if constexpr (F == kFmtUnit8)
     load_vals8<float>(val + p, v);
   else
     load_vals_cs<float>(val + p, v);
@@ -59,20 +71,21 @@ __device__ __forceinline__ void chunk_vals(const VT* val, int32_t p, float (&v)[
 
 // Product of CSR row `row` with right-hand side r of the interleaved xi, in
 // the chunk order of the single-vector default shape (16 lanes).
-template <typename VT, int RS, bool CMP>
+template <typename VT, int RS, int F>
 __device__ __forceinline__ float row_dot_rhs(int64_t row, const int32_t* __restrict__ rp,
                                              const int32_t* __restrict__ rl, const ColIdx ci,
                                              const VT* __restrict__ val,
                                              const float* __restrict__ xi, int r, int gl) {
-  constexpr int C = CMP ? 8 : 4;
+  constexpr int C = kFmtChunk<F>;
   constexpr int S = kGroup * C;
   const int32_t start = __ldg(rp + row), len = __ldg(rl + row);
+  const int32_t blk = F == kFmtBlock4 ? __ldg(ci.rblk + row) : 0;
   float acc = 0.f;
   for (int32_t e = gl * C; e < len; e += S) {
     int32_t c[C];
     float v[C];
-    chunk_cols<CMP>(ci, start + e, c);
-    chunk_vals<VT, CMP>(val, start + e, v);
+    chunk_cols<F>(ci, start + e, e, blk, c);
+    chunk_vals<VT, F>(val, start + e, v);
 #pragma unroll
     for (int i = 0; i < C; ++i) acc = fmaf(v[i], __ldg(xi + (int64_t)c[i] * RS + r), acc);
   }
@@ -92,18 +105,18 @@ __device__ __forceinline__ void gather_rhs(const float* __restrict__ xi, int32_t
 // y[r * ystride + row] = (A xi_r)(row) for r < R, rows of the shared CSR;
 // pivot blocks as in k_spmv_pivots, with output rows of problem p at
 // p * ystride + row.
-template <typename VT, int RS, bool CMP>
+template <typename VT, int RS, int F>
 __global__ void __launch_bounds__(256, 4)
     k_spmm_pivots(int64_t rows, const int32_t* __restrict__ rp, const int32_t* __restrict__ rl,
                   const ColIdx ci, const VT* __restrict__ val, const float* __restrict__ xi,
                   float* __restrict__ y, int64_t ystride, int R, PivotCoef pc) {
-  constexpr int C = CMP ? 8 : 4;
+  constexpr int C = kFmtChunk<F>;
   constexpr int S = kGroup * C;
   const int lane = threadIdx.x & 31;
   const int npiv_all = pc.npiv_blocks * pc.nprob;
   if ((int)blockIdx.x < npiv_all) {
     pivot_blocks<float, kGroup>(pc, [=](int p, int32_t row, int gl) {
-      return row_dot_rhs<VT, RS, CMP>((int64_t)row - (int64_t)p * ystride, rp, rl, ci, val, xi,
+      return row_dot_rhs<VT, RS, F>((int64_t)row - (int64_t)p * ystride, rp, rl, ci, val, xi,
                                       p, gl);
     });
     return;
@@ -115,14 +128,15 @@ __global__ void __launch_bounds__(256, 4)
   const int gl = lane & (kGroup - 1);
   const int32_t start = valid ? __ldg(rp + row) : 0;
   const int32_t len = valid ? __ldg(rl + row) : 0;
+  const int32_t blk = F == kFmtBlock4 && valid ? __ldg(ci.rblk + row) : 0;
   float acc[RS];
 #pragma unroll
   for (int r = 0; r < RS; ++r) acc[r] = 0.f;
   for (int32_t e = gl * C; e < len; e += S) {
     int32_t cs[C];
     float v[C];
-    chunk_cols<CMP>(ci, start + e, cs);
-    chunk_vals<VT, CMP>(val, start + e, v);
+    chunk_cols<F>(ci, start + e, e, blk, cs);
+    chunk_vals<VT, F>(val, start + e, v);
 #pragma unroll
     for (int i = 0; i < C; ++i) {
       float xv[RS];
@@ -244,28 +258,45 @@ cudaError_t upload_padded(int64_t rows, int64_t cols, const std::vector<int64_t>
   if (tot && (e = cudaMemcpyAsync(out->col, pc.data(), tot * sizeof(int32_t),
                                   cudaMemcpyHostToDevice, s)) != cudaSuccess)
     return e;
-  // 16-bit column offsets when every 8-entry unit (rows start and end on unit
-  // boundaries) spans fewer than 2^16 columns: offset = column - unit minimum
+  // 16-bit column offsets, from the smallest column of every 64-entry block of
+  // a row when each block spans fewer than 2^16 columns, else from that of
+  // every 8-entry unit (rows start and end on unit boundaries) when those do
   const int64_t units = tot / kRowAlign;
   std::vector<uint16_t> po;
-  std::vector<int32_t> pb;
-  bool fits = units > 0;
+  std::vector<int32_t> pb, bb, rb;
+  auto span = [&](int64_t a, int64_t b, int32_t& lo) {
+    int32_t hi = lo = pc[a];
+    for (int64_t q = a + 1; q < b; ++q) {
+      lo = std::min(lo, pc[q]);
+      hi = std::max(hi, pc[q]);
+    }
+    return (int64_t)hi - lo <= 65535;
+  };
+  auto fill = [&](int64_t a, int64_t b, int32_t lo) {
+    for (int64_t q = a; q < b; ++q) po[q] = (uint16_t)(pc[q] - lo);
+    for (int64_t u = a / kRowAlign; u < b / kRowAlign; ++u) pb[u] = lo;
+  };
+  bool fits = units > 0, blocks_fit = units > 0;
   if (fits) {
     po.resize((size_t)tot);
     pb.resize((size_t)units);
-    for (int64_t u = 0; u < units && fits; ++u) {
-      const int32_t* c = pc.data() + u * kRowAlign;
-      int32_t lo = c[0], hi = c[0];
-      for (int i = 1; i < kRowAlign; ++i) {
-        lo = std::min(lo, c[i]);
-        hi = std::max(hi, c[i]);
+    rb.resize((size_t)rows);
+    for (int64_t r = 0; r < rows && blocks_fit; ++r) {
+      rb[r] = (int32_t)bb.size();
+      for (int64_t a = prp[r]; a < prp[r] + prl[r] && blocks_fit; a += kPermBlock) {
+        const int64_t b = std::min<int64_t>(a + kPermBlock, prp[r] + prl[r]);
+        int32_t lo;
+        blocks_fit = span(a, b, lo);
+        if (blocks_fit) {
+          fill(a, b, lo);
+          bb.push_back(lo);
+        }
       }
-      if ((int64_t)hi - lo > 65535) {
-        fits = false;
-        break;
-      }
-      pb[u] = lo;
-      for (int i = 0; i < kRowAlign; ++i) po[u * kRowAlign + i] = (uint16_t)(c[i] - lo);
+    }
+    for (int64_t u = 0; u < units && fits && !blocks_fit; ++u) {
+      int32_t lo;
+      fits = span(u * kRowAlign, (u + 1) * kRowAlign, lo);
+      if (fits) fill(u * kRowAlign, (u + 1) * kRowAlign, lo);
     }
   }
   if (fits) {
@@ -280,8 +311,19 @@ cudaError_t upload_padded(int64_t rows, int64_t cols, const std::vector<int64_t>
     if ((e = cudaMemcpyAsync(out->ubase, pb.data(), nub * sizeof(int32_t),
                              cudaMemcpyHostToDevice, s)) != cudaSuccess)
       return e;
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;  // po, pb go out of scope
+    if (blocks_fit) {
+      if ((e = cudaMalloc(&out->bbase, bb.size() * sizeof(int32_t))) != cudaSuccess) return e;
+      if ((e = cudaMalloc(&out->rblk, rows * sizeof(int32_t))) != cudaSuccess) return e;
+      if ((e = cudaMemcpyAsync(out->bbase, bb.data(), bb.size() * sizeof(int32_t),
+                               cudaMemcpyHostToDevice, s)) != cudaSuccess)
+        return e;
+      if ((e = cudaMemcpyAsync(out->rblk, rb.data(), rows * sizeof(int32_t),
+                               cudaMemcpyHostToDevice, s)) != cudaSuccess)
+        return e;
+    }
+    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;  // po, pb.. go out of scope
     out->compressed = 1;
+    out->block_compressed = blocks_fit;
   }
   if (tot) {
     if (vt == LSLU_F64) {
@@ -328,6 +370,10 @@ cudaError_t build_csr_pair(int64_t m, int64_t n, const int64_t* rp, const int32_
     }
   const cudaError_t e2 = upload_padded(n, m, rpt, cit, vt_, vt, AT, s);
   A->shape = AT->shape = default_shape(vt);
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess)
+    cudaDeviceGetAttribute(&A->num_sms, cudaDevAttrMultiProcessorCount, dev);
+  AT->num_sms = A->num_sms;
   return e2;
 }
 
@@ -338,6 +384,8 @@ void free_csr(DevCsr* c) {
   cudaFree(c->val);
   cudaFree(c->off);
   cudaFree(c->ubase);
+  cudaFree(c->bbase);
+  cudaFree(c->rblk);
   *c = DevCsr();
 }
 
@@ -357,6 +405,14 @@ bool native(int vt) {
 
 }  // namespace
 
+// Entries (with padding) from which the default FP32 / BF16 products read
+// 16-bit offsets with four chunks in flight (stream_rows).  Below, the matrix
+// stays in L2 and a product is a few dependent round trips, where the extra
+// base read and the wider step cost more than the bytes: a pair of products
+// 8.2 us either way up to 0.4 M entries, 12.4 against 14.6 us at 1.35 M, 18.4
+// against 22.0 at 3.2 M; a 32x32 solve (0.05 M) 2.20 against 2.15 ms.
+constexpr int64_t kStreamMinEntries = 1 << 20;
+
 // Native products (FP64 vectors for FP64 values, FP32 otherwise) run in the
 // matrix's shape and column format; the others (FP64 vectors on FP32 / BF16
 // values: r0 with x0, the adjoint's x0 term) in the default shape.
@@ -366,12 +422,21 @@ void launch_spmv(const DevCsr& A, int vt, const XT* x, YT* y, cudaStream_t s, in
     launch_spmv_shape(A.shape, A, vt, x, y, s);
     return;
   }
+  if constexpr (std::is_same<XT, float>::value) {
+    if (A.nnz_padded >= kStreamMinEntries) {
+      if (vt == LSLU_F32)
+        spmv_run<float, XT, YT, 16, 4, true>(A, x, y, s);
+      else
+        spmv_run<__nv_bfloat16, XT, YT, 16, 4, true>(A, x, y, s);
+      return;
+    }
+  }
   if (vt == LSLU_F64)
-    spmv_run<double, XT, YT, 16, 1, false>(A, x, y, s);
+    spmv_run<double, XT, YT, 16, 1>(A, x, y, s);
   else if (vt == LSLU_F32)
-    spmv_run<float, XT, YT, 16, 2, false>(A, x, y, s);
+    spmv_run<float, XT, YT, 16, 2>(A, x, y, s);
   else
-    spmv_run<__nv_bfloat16, XT, YT, 16, 2, false>(A, x, y, s);
+    spmv_run<__nv_bfloat16, XT, YT, 16, 2>(A, x, y, s);
 }
 
 template <typename XT, typename YT>
@@ -382,12 +447,21 @@ void launch_spmv_pivots(const DevCsr& A, int vt, const XT* x, YT* y, PivotCoef p
     launch_spmv_pivots_shape(A.shape, A, vt, x, y, pc, s);
     return;
   }
+  if constexpr (std::is_same<XT, float>::value) {
+    if (A.nnz_padded >= kStreamMinEntries) {
+      if (vt == LSLU_F32)
+        spmv_pivots_run<float, XT, YT, 16, 4, true>(A, x, y, pc, s);
+      else
+        spmv_pivots_run<__nv_bfloat16, XT, YT, 16, 4, true>(A, x, y, pc, s);
+      return;
+    }
+  }
   if (vt == LSLU_F64)
-    spmv_pivots_run<double, XT, YT, 16, 1, false>(A, x, y, pc, s);
+    spmv_pivots_run<double, XT, YT, 16, 1>(A, x, y, pc, s);
   else if (vt == LSLU_F32)
-    spmv_pivots_run<float, XT, YT, 16, 2, false>(A, x, y, pc, s);
+    spmv_pivots_run<float, XT, YT, 16, 2>(A, x, y, pc, s);
   else
-    spmv_pivots_run<__nv_bfloat16, XT, YT, 16, 2, false>(A, x, y, pc, s);
+    spmv_pivots_run<__nv_bfloat16, XT, YT, 16, 2>(A, x, y, pc, s);
 }
 
 template <typename VT, int RS>
@@ -395,14 +469,15 @@ void spmm_typed(const DevCsr& A, const float* xi, float* y, int64_t ystride, int
                 const PivotCoef& pc, cudaStream_t s) {
   const int64_t blocks =
       (int64_t)pc.npiv_blocks * pc.nprob + (A.rows + kRowsPerBlock - 1) / kRowsPerBlock;
-  const ColIdx ci{A.col, A.off, A.ubase};
   const VT* v = reinterpret_cast<const VT*>(A.val);
-  if (A.compressed && A.use_cmp)
-    k_spmm_pivots<VT, RS, true><<<(unsigned)blocks, 256, 0, s>>>(A.rows, A.row_ptr, A.row_len,
-                                                                 ci, v, xi, y, ystride, R, pc);
+  auto run = [&](auto F) {
+    k_spmm_pivots<VT, RS, F.value><<<(unsigned)blocks, 256, 0, s>>>(
+        A.rows, A.row_ptr, A.row_len, col_idx(A), v, xi, y, ystride, R, pc);
+  };
+  if (A.nnz_padded >= kStreamMinEntries && !A.use_cmp)
+    with_format<true>(A, run);
   else
-    k_spmm_pivots<VT, RS, false><<<(unsigned)blocks, 256, 0, s>>>(A.rows, A.row_ptr, A.row_len,
-                                                                  ci, v, xi, y, ystride, R, pc);
+    with_format<false>(A, run);
 }
 
 template <typename VT>

@@ -16,10 +16,27 @@
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "lslu_internal.cuh"
 
 namespace lslu {
 namespace {
+
+// The default FP32 / BF16 products run kStreamBlocksPerSm blocks per SM with
+// four chunks in flight per lane (64 registers) and hand every block several
+// row groups.  What bounds them is how many loads an SM keeps in flight: the
+// matrix stream alone (no gathers) takes 113 us on the renumbered 512x512 CT
+// matrix (728 MB), a gather that always hits one L1 sector adds 15 us, its
+// real locality 4 us more.  Measured there, A / A^T in us (events around a
+// product after an L2 flush, ~6 us of which are the events and the launch):
+// 157.6 / 153.6 on 32-bit columns, two chunks, 6 blocks per SM; 135.2 / 133.1
+// the same on block offsets; 131 / 127 with four chunks and 4 blocks;
+// 125.0 / 120.8 with 4 resident blocks per SM taking the row groups in turn
+// (no block starts, the next group's row pointers read ahead).  Two chunks
+// with resident blocks (147-176), register-staged prefetching (129-150) and
+// bulk L2 prefetches ahead of the blocks (129-141) were slower.
+constexpr int kStreamBlocksPerSm = 4;
 
 template <typename VT>
 struct ValTraits {
@@ -31,6 +48,13 @@ struct ValTraits {
 template <typename VT, int E>
 constexpr int min_blocks() {
   return (E >= 2 || sizeof(VT) == 8) ? 6 : 8;
+}
+
+template <typename VT, int G, int U, int F>
+constexpr int resident_blocks() {
+  if (G == 0) return sizeof(VT) == 8 && U > 4 ? 4 : min_blocks<VT, U / 4>();
+  if (U >= 4) return kStreamBlocksPerSm;
+  return min_blocks<VT, F == 1 /* 8-entry chunks */ ? 2 * U : U>();
 }
 
 template <typename AT>
@@ -119,13 +143,27 @@ __device__ __forceinline__ void load_vals8(const __nv_bfloat16* p, AT (&v)[8]) {
   }
 }
 
-// The column storage a kernel reads: 32-bit indices (chunks of 4 entries) or,
-// when every 8-entry unit spans fewer than 2^16 columns, 16-bit offsets from
-// the unit's first column (chunks of 8 entries; 2.5 bytes per entry).
+// 4 16-bit offsets of one 4-entry chunk (8 bytes).
+__device__ __forceinline__ uint2 ld_stream_off4(const uint16_t* p) {
+  uint2 c;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.u32 {%0,%1}, [%2];"
+               : "=r"(c.x), "=r"(c.y)
+               : "l"(p));
+  return c;
+}
+
+// The column storage a kernel reads (Fmt): 32-bit indices (chunks of 4
+// entries), or 16-bit offsets from the smallest column of their 8-entry unit,
+// in chunks of 8 entries (the /16-bit shapes) or of 4 (the default shape: the
+// chunks, and so the sums, of the 32-bit format bit for bit), or offsets from
+// the smallest column of their 64-entry block, in chunks of 4.
+enum Fmt { kFmtCol = 0, kFmtUnit8 = 1, kFmtUnit4 = 2, kFmtBlock4 = 3 };
 struct ColIdx {
   const int32_t* col;     // nnz_padded 32-bit columns
   const uint16_t* off;    // nnz_padded offsets (compressed)
   const int32_t* ubase;   // nnz_padded / 8 unit bases (compressed)
+  const int32_t* bbase;   // block bases (block-compressed)
+  const int32_t* rblk;    // first block of every row
 };
 
 // Dot product of one CSR row with x, computed by one group of G lanes (result
@@ -213,6 +251,52 @@ __device__ __forceinline__ YT row_dot_len(int32_t start, int32_t len,
   return group_sum<G>(acc);
 }
 
+// row_dot_len on 16-bit offsets: the same chunks, order and butterfly, so the
+// same bits, from 2.5 (kFmtUnit4) or 2.06 (kFmtBlock4) instead of 4 bytes of
+// column storage per entry.
+template <typename VT, typename XT, typename YT, int G, int U, int F>
+__device__ __forceinline__ YT row_dot_len_h(int32_t start, int32_t len, int32_t blk,
+                                            const ColIdx ci, const VT* __restrict__ val,
+                                            const XT* __restrict__ x, int gl) {
+  constexpr int C = ValTraits<VT>::kChunk;
+  constexpr int S = G * C;
+  static_assert(F == kFmtUnit4 || (F == kFmtBlock4 && S == kPermBlock), "one block per chunk step");
+  YT acc = 0;
+  for (int32_t e = gl * C; e < len; e += U * S) {
+    int32_t cidx[U][C];
+    YT v[U][C];
+    bool has[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      has[u] = u == 0 || e + u * S < len;
+      if (has[u]) {
+        const int32_t p = start + e + u * S;
+        const uint2 o = ld_stream_off4(ci.off + p);
+        const int32_t b = F == kFmtBlock4 ? __ldg(ci.bbase + blk + (e + u * S) / kPermBlock)
+                                          : __ldg(ci.ubase + (p >> 3));
+        cidx[u][0] = b + (int32_t)(o.x & 0xffffu);
+        cidx[u][1] = b + (int32_t)(o.x >> 16);
+        cidx[u][2] = b + (int32_t)(o.y & 0xffffu);
+        cidx[u][3] = b + (int32_t)(o.y >> 16);
+        load_vals_cs<YT>(val + p, v[u]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < C; ++i) v[u][i] = 0;
+      }
+    }
+    XT xv[U][C];
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int i = 0; i < C; ++i) xv[u][i] = has[u] ? __ldg(x + cidx[u][i]) : (XT)0;
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int i = 0; i < C; ++i) acc = fma(v[u][i], (YT)xv[u][i], acc);
+  }
+  return group_sum<G>(acc);
+}
+
 // Scalar stream loads (one entry per lane) without L1 allocation.
 __device__ __forceinline__ float ld_stream1(const float* p) {
   float v;
@@ -275,37 +359,72 @@ __device__ __forceinline__ YT row_dot_s1(int32_t start, int32_t len, const ColId
   return group_sum<32>(acc);
 }
 
-// G = 0 selects the warp-per-row stride-1 form (row_dot_s1) with U entries in
-// flight per lane.
-template <typename VT, typename XT, typename YT, int G, int U, bool CMP>
-__device__ __forceinline__ YT row_dot(int64_t row, bool valid, const int32_t* __restrict__ rp,
-                                      const int32_t* __restrict__ rl, const ColIdx ci,
-                                      const VT* __restrict__ val, const XT* __restrict__ x,
-                                      int gl) {
-  const int32_t start = valid ? __ldg(rp + row) : 0;
-  const int32_t len = valid ? __ldg(rl + row) : 0;
-  if constexpr (G == 0)
-    return row_dot_s1<VT, XT, YT, U, CMP>(start, len, ci, val, x, gl);
-  else if constexpr (CMP)
-    return row_dot_len_c<VT, XT, YT, G, U>(start, len, ci, val, x, gl);
-  else
-    return row_dot_len<VT, XT, YT, G, U>(start, len, ci.col, val, x, gl);
+// Where a row is stored: first entry, padded length and first block (an empty
+// row past the end of the matrix).
+struct RowAt {
+  int32_t start, len, blk;
+};
+template <int F>
+__device__ __forceinline__ RowAt row_at(int64_t row, bool valid, const int32_t* __restrict__ rp,
+                                        const int32_t* __restrict__ rl, const ColIdx& ci) {
+  RowAt r;
+  r.start = valid ? __ldg(rp + row) : 0;
+  r.len = valid ? __ldg(rl + row) : 0;
+  r.blk = F == kFmtBlock4 && valid ? __ldg(ci.rblk + row) : 0;
+  return r;
 }
 
-template <typename VT, typename XT, typename YT, int G, int U, bool CMP>
-__global__ void __launch_bounds__(256, (G == 0 && sizeof(VT) == 8 && U > 4) ? 4 : min_blocks<VT, G == 0 ? U / 4 : (CMP ? 2 * U : U)>())
+// G = 0 selects the warp-per-row stride-1 form (row_dot_s1) with U entries in
+// flight per lane.
+template <typename VT, typename XT, typename YT, int G, int U, int F>
+__device__ __forceinline__ YT row_dot(const RowAt& r, const ColIdx ci, const VT* __restrict__ val,
+                                      const XT* __restrict__ x, int gl) {
+  if constexpr (G == 0)
+    return row_dot_s1<VT, XT, YT, U, F == kFmtUnit8>(r.start, r.len, ci, val, x, gl);
+  else if constexpr (F == kFmtUnit8)
+    return row_dot_len_c<VT, XT, YT, G, U>(r.start, r.len, ci, val, x, gl);
+  else if constexpr (F == kFmtUnit4 || F == kFmtBlock4)
+    return row_dot_len_h<VT, XT, YT, G, U, F>(r.start, r.len, r.blk, ci, val, x, gl);
+  else
+    return row_dot_len<VT, XT, YT, G, U>(r.start, r.len, ci.col, val, x, gl);
+}
+
+// The rows of block b of nb (row groups b, b + nb, ... of 256 / GL rows): y =
+// A x on them, with the next group's row pointers read ahead.
+template <typename VT, typename XT, typename YT, int G, int U, int F>
+__device__ __forceinline__ void stream_rows(int64_t b, int64_t nb, int64_t rows,
+                                            const int32_t* __restrict__ rp,
+                                            const int32_t* __restrict__ rl, const ColIdx ci,
+                                            const VT* __restrict__ val,
+                                            const XT* __restrict__ x, YT* __restrict__ y) {
+  constexpr int GL = G == 0 ? 32 : G;  // lanes per row
+  constexpr int RPB = 256 / GL;        // rows per group
+  const int gl = threadIdx.x & (GL - 1);
+  const int in_warp = (threadIdx.x & 31) / GL;  // this lane's row among its warp's
+  const int64_t stride = nb * RPB;
+  int64_t row = b * RPB + threadIdx.x / GL;
+  if (row - in_warp >= rows) return;  // the whole warp is past the last row
+  RowAt r = row_at<F>(row, row < rows, rp, rl, ci);
+  while (true) {
+    const int64_t next = row + stride;
+    // (the same for the whole warp; the other shapes have one group per block)
+    const bool more = U >= 4 && G != 0 && next - in_warp < rows;
+    RowAt rn = {0, 0, 0};
+    if (more) rn = row_at<F>(next, next < rows, rp, rl, ci);
+    const YT acc = row_dot<VT, XT, YT, G, U, F>(r, ci, val, x, gl);
+    if (row < rows && gl == 0) y[row] = acc;
+    if (!more) return;
+    row = next;
+    r = rn;
+  }
+}
+
+template <typename VT, typename XT, typename YT, int G, int U, int F>
+__global__ void __launch_bounds__(256, (resident_blocks<VT, G, U, F>()))
     k_spmv(int64_t rows, const int32_t* __restrict__ rp, const int32_t* __restrict__ rl,
            const ColIdx ci, const VT* __restrict__ val, const XT* __restrict__ x,
            YT* __restrict__ y) {
-  constexpr int GL = G == 0 ? 32 : G;  // lanes per row
-  constexpr int RPB = 256 / GL;        // rows per block
-  const int gl = threadIdx.x & (GL - 1);
-  const int64_t row = (int64_t)blockIdx.x * RPB + threadIdx.x / GL;
-  if ((int64_t)blockIdx.x * RPB + (threadIdx.x & ~31) / GL >= rows)
-    return;  // the whole warp is past the last row
-  const bool valid = row < rows;
-  const YT acc = row_dot<VT, XT, YT, G, U, CMP>(row, valid, rp, rl, ci, val, x, gl);
-  if (valid && gl == 0) y[row] = acc;
+  stream_rows<VT, XT, YT, G, U, F>(blockIdx.x, gridDim.x, rows, rp, rl, ci, val, x, y);
 }
 
 // y = A x plus the elimination coefficients of the next Hessenberg step,
@@ -385,68 +504,81 @@ __device__ __forceinline__ void pivot_blocks(const PivotCoef& pc, RowDot rowdot)
   }
 }
 
-template <typename VT, typename XT, typename YT, int G, int U, bool CMP>
-__global__ void __launch_bounds__(256, (G == 0 && sizeof(VT) == 8 && U > 4) ? 4 : min_blocks<VT, G == 0 ? U / 4 : (CMP ? 2 * U : U)>())
+template <typename VT, typename XT, typename YT, int G, int U, int F>
+__global__ void __launch_bounds__(256, (resident_blocks<VT, G, U, F>()))
     k_spmv_pivots(int64_t rows, const int32_t* __restrict__ rp, const int32_t* __restrict__ rl,
                   const ColIdx ci, const VT* __restrict__ val, const XT* __restrict__ x,
                   YT* __restrict__ y, PivotCoef pc) {
-  constexpr int GL = G == 0 ? 32 : G;
-  constexpr int RPB = 256 / GL;
   pdl_wait();  // x and the pivot rows come from the kernels before
   pdl_trigger();
-  const int lane = threadIdx.x & 31;
   const int npiv_all = pc.npiv_blocks * pc.nprob;
   if ((int)blockIdx.x >= npiv_all) {  // streaming rows (all but the first npiv_all blocks)
-    const int64_t b0 = (int64_t)(blockIdx.x - npiv_all) * RPB;
-    if (b0 + (threadIdx.x & ~31) / GL >= rows) return;  // whole warp past the end
-    const int64_t row = b0 + threadIdx.x / GL;
-    const bool valid = row < rows;
-    const YT acc =
-        row_dot<VT, XT, YT, G, U, CMP>(row, valid, rp, rl, ci, val, x, lane & (GL - 1));
-    if (valid && (lane & (GL - 1)) == 0) y[row] = acc;
+    stream_rows<VT, XT, YT, G, U, F>(blockIdx.x - npiv_all, gridDim.x - npiv_all, rows, rp, rl, ci,
+                                     val, x, y);
     return;
   }
-  pivot_blocks<YT, GL>(pc, [=](int, int32_t row, int gl) {
-    return row_dot<VT, XT, YT, G, U, CMP>(row, true, rp, rl, ci, val, x, gl);
+  pivot_blocks<YT, G == 0 ? 32 : G>(pc, [=](int, int32_t row, int gl) {
+    return row_dot<VT, XT, YT, G, U, F>(row_at<F>(row, true, rp, rl, ci), ci, val, x, gl);
   });
 }
 
-// Launch in the matrix's column format: 16-bit offsets when its shape reads
-// them (use_cmp) and MAYCMP (native vector types), else 32-bit columns.
-template <typename VT, typename XT, typename YT, int G, int U, bool MAYCMP = true>
-void spmv_run(const DevCsr& A, const XT* x, YT* y, cudaStream_t s) {
-  if (A.rows == 0) return;
-  constexpr int GL = G == 0 ? 32 : G;
-  const int64_t blocks = (A.rows + 256 / GL - 1) / (256 / GL);
-  const ColIdx ci{A.col, A.off, A.ubase};
-  const VT* v = reinterpret_cast<const VT*>(A.val);
-  if constexpr (MAYCMP) {
-    if (A.compressed && A.use_cmp) {
-      k_spmv<VT, XT, YT, G, U, true><<<(unsigned)blocks, 256, 0, s>>>(A.rows, A.row_ptr,
-                                                                       A.row_len, ci, v, x, y);
-      return;
-    }
+// Calls f with the column format to launch as a compile-time constant.
+// Shapes of the /16-bit list read 8-entry units; DEF marks the default shape,
+// which reads 16-bit offsets wherever the matrix has them.
+template <bool DEF, typename Fn>
+void with_format(const DevCsr& A, Fn f) {
+  if constexpr (DEF) {
+    if (A.block_compressed)
+      f(std::integral_constant<int, kFmtBlock4>{});
+    else if (A.compressed)
+      f(std::integral_constant<int, kFmtUnit4>{});
+    else
+      f(std::integral_constant<int, kFmtCol>{});
+  } else {
+    if (A.compressed && A.use_cmp)
+      f(std::integral_constant<int, kFmtUnit8>{});
+    else
+      f(std::integral_constant<int, kFmtCol>{});
   }
-  k_spmv<VT, XT, YT, G, U, false><<<(unsigned)blocks, 256, 0, s>>>(A.rows, A.row_ptr,
-                                                                    A.row_len, ci, v, x, y);
 }
 
-template <typename VT, typename XT, typename YT, int G, int U, bool MAYCMP = true>
-void spmv_pivots_run(const DevCsr& A, const XT* x, YT* y, const PivotCoef& pc, cudaStream_t s) {
-  constexpr int GL = G == 0 ? 32 : G;
-  const int64_t blocks =
-      (int64_t)pc.npiv_blocks * pc.nprob + (A.rows + 256 / GL - 1) / (256 / GL);
-  const ColIdx ci{A.col, A.off, A.ubase};
+inline ColIdx col_idx(const DevCsr& A) { return {A.col, A.off, A.ubase, A.bbase, A.rblk}; }
+
+// Streaming blocks of a product beside npiv pivot blocks: one per row group,
+// or (U = 4: the default FP32 / BF16 products) as many as are resident next to
+// the pivot blocks, each taking several groups.  Where the pivot blocks of a
+// batch alone fill half the GPU, blocks of two groups instead: resident blocks
+// of equal shares would wait for the ones that start late.
+template <int U>
+int64_t stream_blocks(const DevCsr& A, int64_t groups, int64_t npiv) {
+  if (U < 4 || A.num_sms <= 0) return groups;
+  const int64_t slots = (int64_t)A.num_sms * kStreamBlocksPerSm;
+  const int64_t nb = npiv <= slots / 2 ? slots - npiv : (groups + 1) / 2;
+  return groups < nb ? groups : nb;
+}
+
+template <typename VT, typename XT, typename YT, int G, int U, bool DEF = false>
+void spmv_run(const DevCsr& A, const XT* x, YT* y, cudaStream_t s) {
+  if (A.rows == 0) return;
+  constexpr int RPB = 256 / (G == 0 ? 32 : G);
+  const int64_t blocks = stream_blocks<U>(A, (A.rows + RPB - 1) / RPB, 0);
   const VT* v = reinterpret_cast<const VT*>(A.val);
-  if constexpr (MAYCMP) {
-    if (A.compressed && A.use_cmp) {
-      launch_pdl(k_spmv_pivots<VT, XT, YT, G, U, true>, dim3((unsigned)blocks), dim3(256), 0, s,
-                 A.rows, A.row_ptr, A.row_len, ci, v, x, y, pc);
-      return;
-    }
-  }
-  launch_pdl(k_spmv_pivots<VT, XT, YT, G, U, false>, dim3((unsigned)blocks), dim3(256), 0, s,
-             A.rows, A.row_ptr, A.row_len, ci, v, x, y, pc);
+  with_format<DEF>(A, [&](auto F) {
+    k_spmv<VT, XT, YT, G, U, F.value><<<(unsigned)blocks, 256, 0, s>>>(
+        A.rows, A.row_ptr, A.row_len, col_idx(A), v, x, y);
+  });
+}
+
+template <typename VT, typename XT, typename YT, int G, int U, bool DEF = false>
+void spmv_pivots_run(const DevCsr& A, const XT* x, YT* y, const PivotCoef& pc, cudaStream_t s) {
+  constexpr int RPB = 256 / (G == 0 ? 32 : G);
+  const int64_t npiv = (int64_t)pc.npiv_blocks * pc.nprob;
+  const int64_t blocks = npiv + stream_blocks<U>(A, (A.rows + RPB - 1) / RPB, npiv);
+  const VT* v = reinterpret_cast<const VT*>(A.val);
+  with_format<DEF>(A, [&](auto F) {
+    launch_pdl(k_spmv_pivots<VT, XT, YT, G, U, F.value>, dim3((unsigned)blocks), dim3(256), 0, s,
+               A.rows, A.row_ptr, A.row_len, col_idx(A), v, x, y, pc);
+  });
 }
 
 }  // namespace
