@@ -22,7 +22,10 @@
 //      T (order 2k+1, zero diagonal, off-diagonals alpha_0, beta_1, alpha_1,
 //      ..., beta_k).  Sturm counts at 32 points per round (one per lane,
 //      geometric spacing while the bracket spans more than an octave) shrink
-//      the bracket of sigma_i 33-fold per round.  c = beta U^T e1 (Eq. gcv2):
+//      the bracket of sigma_i 33-fold per round until four points around it
+//      are close; from there the zero of the cubic through their determinants
+//      is the centre of the next round's points, 2^-51 to 2^-8 of it away.
+//      c = beta U^T e1 (Eq. gcv2):
 //      since P e1 = e1, c_i^2 is 2 beta^2 times the squared first component of
 //      T's eigenvector for sigma_i, the residue of e1^T (T - theta)^-1 e1 =
 //      det(T_{2:,2:} - theta) / det(T - theta), with the leading and trailing
@@ -148,22 +151,37 @@ __device__ __forceinline__ void house(double x0, double ss, double& tau, double&
   scale = neg ? -id : id;
 }
 
+// The lambda grid, sigma_1 10^(-14 + t / 16), t = 0 .. 256: a decade times a
+// sixteenth of one (an FP64 pow takes about 3 us here).
+__constant__ double kDecade[17] = {1e-14, 1e-13, 1e-12, 1e-11, 1e-10, 1e-9, 1e-8, 1e-7, 1e-6,
+                                   1e-5,  1e-4,  1e-3,  1e-2,  1e-1,  1.0,  1e1,  1e2};
+__constant__ double kSixteenth[16] = {
+    1.0,                1.1547819846894582, 1.333521432163324,  1.539926526059492,
+    1.7782794100389228, 2.053525026457146,  2.3713737056616555, 2.738419634264361,
+    3.1622776601683795, 3.651741272548377,  4.216965034285822,  4.869675251658631,
+    5.623413251903491,  6.493816315762113,  7.498942093324558,  8.659643233600654};
+__device__ __forceinline__ double grid_lambda(double s1, int t) {
+  return s1 * (kDecade[t >> 4] * kSixteenth[t & 15]);
+}
+
 // Squared off-diagonals t_j^2 of the Golub-Kahan tridiagonal T (1-based j,
 // t_j couples rows j and j+1): t_{2i+1} = alpha_i, t_{2i+2} = beta_{i+1}.
 // The recurrences below read t2[j]; the FP64 pipe is the scarce resource on
-// this GPU, so signs and zero tests use integer operations on the bits and
-// the over/underflow check runs once every 8 steps (|p| grows by at most a
-// factor (|theta| + 2 max|t|)^8 < 2^160 between checks for the matrices
-// solved here, far inside the 2^+-400 rescaling margin).
-__device__ __forceinline__ int sign_change(double a, double b) {
-  const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
-  // a change, or an exact zero (which counts as a change)
-  return (int)(((ia ^ ib) < 0) | ((ia << 1) == 0));
+// this GPU, so signs and scales are handled on the bits, and the
+// over/underflow check runs once every 8 steps (T is scaled to max |t| < 1,
+// so |p| grows by less than 3^8 between checks, far inside the 2^+-400
+// rescaling margin).
+__device__ __forceinline__ int biased_exponent(double x) {
+  return (int)((__double_as_longlong(x) >> 52) & 0x7ff);
+}
+// 2^e as a double, -1022 <= e <= 1023.
+__device__ __forceinline__ double pow2(int e) {
+  return __longlong_as_double((long long)(1023 + e) << 52);
 }
 
 __device__ __forceinline__ bool needs_rescale(double p0, double pm1, int& s) {
-  const int e0 = (int)((__double_as_longlong(p0) >> 52) & 0x7ff);
-  const int e1 = (int)((__double_as_longlong(pm1) >> 52) & 0x7ff);
+  const int e0 = biased_exponent(p0);
+  const int e1 = biased_exponent(pm1);
   const int e = e0 > e1 ? e0 : e1;
   if (e > 1023 + 400) {
     s = -400;
@@ -175,38 +193,60 @@ __device__ __forceinline__ bool needs_rescale(double p0, double pm1, int& s) {
   }
   return false;
 }
+// v 2^s on the exponent bits (an FP64 multiplication costs 64 cycles here,
+// ldexp several): exact for normal results, a zero of v's sign below them
+// (the other minor of the pair is then 2^600 larger).
+__device__ __forceinline__ double rescaled(double v, int s) {
+  const int hi = __double2hiint(v), e = (hi >> 20) & 0x7ff;
+  const bool normal = e != 0 && e + s > 0;
+  return __hiloint2double(normal ? hi + s * (1 << 20) : (hi & (int)0x80000000),
+                          normal ? __double2loint(v) : 0);
+}
 
-// Leading-minor recurrence p_j = -theta p_{j-1} - t_{j-1}^2 p_{j-2} of
-// det(T - theta I), optionally with its theta-derivative.  Returns the number
-// of sign changes of p_0..p_n (= eigenvalues of T below theta); p, dp receive
-// the determinant and derivative scaled by 2^-exp2.
 // Number of eigenvalues of T below theta: sign changes along the leading
-// minors p_0 = 1, p_1 = -theta, p_j = -theta p_{j-1} - t_{j-1}^2 p_{j-2}.
+// minors p_0 = 1, p_1 = -theta, p_j = -theta p_{j-1} - t_{j-1}^2 p_{j-2};
+// det receives det(T - theta) scaled by 2^-ex.
 // The product -t_j^2 p_{j-1} of the next step does not depend on p_j; it is
 // issued right after p_j's FMA so that in-order issue does not stall on it
-// (t2[n] must be readable; its value is not used).
-__device__ int sturm_count(const double* t2, int n, double theta) {
+// (t2[n] must be readable; its value is not used).  Two FP64 instructions of
+// 64 cycles per step bound it: 137 cycles per step measured, the sign bits
+// shifted into one word and counted eight at a time (64-bit comparisons per
+// step took 244), T scaled so that the minors rarely leave the 2^400 margins,
+// and rescaled on their exponent bits (ldexp added ~50).
+__device__ int sturm_count(const double* t2, int n, double theta, double& det, int& ex) {
   double pm1 = 1.0, p0 = -theta;
-  int cnt = (int)(__double_as_longlong(p0) < 0);
   double x = -t2[1] * pm1;
+  int cnt = 0, e2 = 0;
+  // sign bits of the last minors, newest lowest (p_0 > 0, p_1); a computed
+  // zero is +0 and counts its one change before or after itself
+  unsigned signs = (unsigned)__double2hiint(p0) >> 31;
+  cnt = (int)signs;
+  auto step = [&](int j) {
+    const double pj = fma(-theta, p0, x);
+    x = -t2[j] * p0;
+    signs = __funnelshift_l((unsigned)__double2hiint(pj), signs, 1);
+    pm1 = p0;
+    p0 = pj;
+  };
   int j = 2;
-  while (j <= n) {
-    const int jend = min(n, j + 7);
-#pragma unroll 4
-    for (; j <= jend; ++j) {
-      const double pj = fma(-theta, p0, x);
-      x = -t2[j] * p0;
-      cnt += sign_change(pj, p0);
-      pm1 = p0;
-      p0 = pj;
-    }
+  for (; j + 7 <= n; j += 8) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) step(j + q);
+    cnt += __popc((signs ^ (signs >> 1)) & 0xffu);
     int sc;
     if (needs_rescale(p0, pm1, sc)) {  // x is proportional to pm1
-      p0 = ldexp(p0, sc);
-      pm1 = ldexp(pm1, sc);
-      x = ldexp(x, sc);
+      p0 = rescaled(p0, sc);
+      pm1 = rescaled(pm1, sc);
+      x = rescaled(x, sc);
+      e2 -= sc;
     }
   }
+  for (; j <= n; ++j) {
+    step(j);
+    cnt += (int)((signs ^ (signs >> 1)) & 1u);
+  }
+  det = p0;
+  ex = e2;
   return cnt;
 }
 
@@ -221,39 +261,38 @@ __device__ void minors(const double* t2, int n, double theta, bool trailing, dou
   // step m (m = 0 ..) uses tt_m = t2[m + 1] (leading) or t2[n - 1 - m]
   // (trailing); the next step's products x = -tt p_{j-1} and
   // z = -tt d_{j-1} - p_j are formed as soon as their inputs exist
-  double pm1 = 1.0, p0 = -theta, dm1 = 0.0, d0 = -1.0;
+  double pm1 = 1.0, p0 = -theta, d0 = -1.0;
   int ex = 0;
   const int stride = trailing ? -1 : 1;
   const double* tp = t2 + (trailing ? n - 1 : 1);
   double x = -tp[0] * pm1;
-  double z = fma(-tp[0], dm1, -p0);
+  double z = -p0;
   const int common = n - 2;  // steps both recurrences take
+  auto step = [&](int m) {
+    const double pj = fma(-theta, p0, x);
+    const double dj = fma(-theta, d0, z);
+    const double tn = tp[(m + 1) * stride];
+    x = -tn * p0;
+    z = fma(-tn, d0, -pj);
+    pm1 = p0;
+    p0 = pj;
+    d0 = dj;
+  };
   int m = 0;
-  while (m < common) {
-    const int mend = min(common, m + 8);
-#pragma unroll 2
-    for (; m < mend; ++m) {
-      const double pj = fma(-theta, p0, x);
-      const double dj = fma(-theta, d0, z);
-      const double tn = tp[(m + 1) * stride];
-      x = -tn * p0;
-      z = fma(-tn, d0, -pj);
-      pm1 = p0;
-      p0 = pj;
-      dm1 = d0;
-      d0 = dj;
-    }
+  for (; m + 8 <= common; m += 8) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) step(m + q);
     int sc;
     if (needs_rescale(p0, pm1, sc)) {  // x and z scale with the minors
-      p0 = ldexp(p0, sc);
-      pm1 = ldexp(pm1, sc);
-      d0 = ldexp(d0, sc);
-      dm1 = ldexp(dm1, sc);
-      x = ldexp(x, sc);
-      z = ldexp(z, sc);
+      p0 = rescaled(p0, sc);
+      pm1 = rescaled(pm1, sc);
+      d0 = rescaled(d0, sc);
+      x = rescaled(x, sc);
+      z = rescaled(z, sc);
       ex -= sc;
     }
   }
+  for (; m < common; ++m) step(m);
   if (!trailing) {  // the leading recurrence has one step more
     const double pj = fma(-theta, p0, x);
     d0 = fma(-theta, d0, z);
@@ -262,6 +301,45 @@ __device__ void minors(const double* t2, int n, double theta, bool trailing, dou
   v = p0;
   dv = d0;
   e = ex;
+}
+
+// The tridiagonal of a problem in shared memory, scaled by a power of two to
+// 1/2 <= max |t| < 1: t2[j] = t_j^2, j = 1..2k (t2[2k+1] = 0 is read, not
+// used, by the last Sturm step); alpha_0..alpha_{k-1} and beta_1..beta_k (at
+// 1..k) unscaled.  Returns 2 max |t| (no eigenvalue of a zero-diagonal
+// tridiagonal reaches it; 0 for a zero matrix), the maximum taken on the bit
+// patterns, and unscale, the power of two that takes scaled values back.
+template <int NW>
+__device__ double load_tridiagonal(const double* al_g, const double* be_g, int k, double* t2,
+                                   double* alv, double* bev, unsigned long long (&gmax)[NW],
+                                   double& unscale) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned long long mx = 0;
+  for (int i = tid; i < k; i += blockDim.x) {
+    const double al = __ldcg(al_g + i), be = __ldcg(be_g + i + 1);
+    alv[i] = al;
+    bev[i + 1] = be;
+    const unsigned long long ba = (unsigned long long)__double_as_longlong(al) & 0x7fffffffffffffffull;
+    const unsigned long long bb = (unsigned long long)__double_as_longlong(be) & 0x7fffffffffffffffull;
+    mx = max(mx, max(ba, bb));
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (lane == 0) gmax[warp] = mx;
+  __syncthreads();
+  for (int q = 0; q < NW; ++q) mx = max(mx, gmax[q]);
+  int shift = 1022 - (int)(mx >> 52);
+  shift = shift > 1000 ? 1000 : shift < -1000 ? -1000 : shift;
+  const double s = pow2(shift);
+  unscale = pow2(-shift);
+  for (int i = tid; i < k; i += blockDim.x) {
+    const double al = alv[i] * s, be = bev[i + 1] * s;
+    t2[2 * i + 1] = al * al;
+    t2[2 * i + 2] = be * be;
+  }
+  if (tid == 0) t2[2 * k + 1] = 0.0;
+  __syncthreads();
+  return 2.0 * s * __longlong_as_double((long long)mx);
 }
 
 // The GCV function (Eqs. gcv2/wgcv) N / D^2 scaled by k and its sign-carrying
@@ -328,9 +406,15 @@ struct Slots {
   double* sig;   // kk+1: singular values, largest first
   double* c2;    // kk+1: c_i^2, then c_{k+1}^2
   double* gv;    // kGrid+1: GCV function on the lambda grid
+  double* gram;  // 6 per group of four right reflectors: their inner products
   double* Qs;    // kk x kk: right reflector j in row j (entries c >= j)
   double* A;     // (kk+1) x kk column slab when shared memory is too small
 };
+
+constexpr int kGroupQ = 4;  // right reflectors applied together (apply_q4)
+__host__ __device__ constexpr int64_t gram_doubles(int64_t kk) {
+  return 6 * ((kk + kGroupQ - 1) / kGroupQ);
+}
 
 __device__ Slots carve(double* base, int kk, int /*CL*/) {
   Slots s;
@@ -341,6 +425,7 @@ __device__ Slots carve(double* base, int kk, int /*CL*/) {
   s.sig = p; p += kk + 1;
   s.c2 = p; p += kk + 1;
   s.gv = p; p += kGrid + 1;
+  s.gram = p; p += gram_doubles(kk);
   s.Qs = p; p += (int64_t)kk * kk;
   s.A = p;
   return s;
@@ -591,26 +676,8 @@ __global__ void __launch_bounds__(kWS * 32) k_sigma(ProjArgs a, ProjWork w) {
   double* bev = alv + K1;     // beta_1..beta_k at 1..k
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = 2 * k + 1;
-  // spectral bound of T: 2 max |t_j| (no eigenvalue of a zero-diagonal
-  // tridiagonal reaches it), the maximum taken on the bit patterns
-  unsigned long long mx = 0;
-  for (int i = tid; i < k; i += blockDim.x) {
-    const double al = ldg_cg(S.al + i), be = ldg_cg(S.be + i + 1);
-    alv[i] = al;
-    bev[i + 1] = be;
-    t2[2 * i + 1] = al * al;
-    t2[2 * i + 2] = be * be;
-    const unsigned long long ba = (unsigned long long)__double_as_longlong(al) & 0x7fffffffffffffffull;
-    const unsigned long long bb = (unsigned long long)__double_as_longlong(be) & 0x7fffffffffffffffull;
-    mx = max(mx, max(ba, bb));
-  }
-  if (tid == 0) t2[2 * k + 1] = 0.0;  // read (not used) by the last Sturm step
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) gmax[warp] = mx;
-  __syncthreads();
-  for (int q = 0; q < kWS; ++q) mx = max(mx, gmax[q]);
-  const double G = 2.0 * __longlong_as_double((long long)mx);
+  double unscale;
+  const double G = load_tridiagonal(S.al, S.be, k, t2, alv, bev, gmax, unscale);
   const int i = i0 + warp;
   if (i > k) return;
   if (i == k) {  // null vector of B^T: u_{i+1} = -alpha_i u_i / beta_{i+1}, u_0 = 1
@@ -634,7 +701,8 @@ __global__ void __launch_bounds__(kWS * 32) k_sigma(ProjArgs a, ProjWork w) {
   // sigma_i, the i-th largest, has target = k-1-i singular values below it;
   // the bracket keeps count(lo) <= target < count(hi), both counts evaluated
   const int target = k - 1 - i;
-  double lo = 0.0, hi = G;
+  double lo = 0.0, hi = G, est = 0.0;
+  bool probe = false;  // est estimates sigma_i inside the bracket
   int rounds = 0;
   if (G > 0.0) {
     const double tiny = G * 0x1p-200;  // below this a singular value is zero
@@ -642,21 +710,57 @@ __global__ void __launch_bounds__(kWS * 32) k_sigma(ProjArgs a, ProjWork w) {
     for (; rounds < 64; ++rounds) {
       if (hi - lo <= 4.0 * kEps * hi || hi <= tiny) break;
       double th;
-      if (lo == 0.0)
+      if (probe) {  // 16 points on each side of est, 2^-51 est .. 2^-8 est away
+        const int q = lane < 16 ? 15 - lane : lane - 16;
+        const unsigned long long exps = q < 8 ? 0x0d0a070503020100ull : 0x2b27231f1b171310ull;
+        const double d = est * pow2(-51 + (int)((exps >> (8 * (q & 7))) & 0xff));
+        th = lane < 16 ? est - d : est + d;
+        th = th < lo ? lo : th > hi ? hi : th;
+      } else if (lo == 0.0) {
         th = hi * exp2(-60.0 * (1.0 - f));  // geometric points down to hi 2^-60
-      else if (hi > 2.0 * lo)
+      } else if (hi > 2.0 * lo) {
         th = lo * exp2(log2(hi / lo) * f);
-      else
+      } else {
         th = fma(hi - lo, f, lo);
-      const int cnt = sturm_count(t2, n, th) - (k + 1);
+      }
+      double det;
+      int ex;
+      const int cnt = sturm_count(t2, n, th, det, ex) - (k + 1);
       const unsigned above = __ballot_sync(0xffffffffu, cnt > target);
       const int fl = above ? __ffs(above) - 1 : 32;  // first point above the target
       const double nhi = __shfl_sync(0xffffffffu, th, fl < 32 ? fl : 0);
       const double nlo = __shfl_sync(0xffffffffu, th, fl > 0 ? fl - 1 : 0);
       const double hi2 = fl < 32 ? nhi : hi, lo2 = fl > 0 ? nlo : lo;
-      if (hi2 == hi && lo2 == lo) break;  // the points no longer split the bracket
+      const bool moved = hi2 != hi || lo2 != lo;
+      if (!moved && !probe) break;  // the points no longer split the bracket
       lo = lo2;
       hi = hi2;
+      probe = false;
+      if (moved && fl >= 2 && fl <= 30) {
+        // sigma_i alone among the four points around it, closely spaced and
+        // with determinants of one scale: the zero of the cubic through
+        // (det, theta), one term of the sum per lane
+        const int b0 = fl - 2, q = lane & 3;
+        const double x0 = __shfl_sync(0xffffffffu, th, b0), x3 = __shfl_sync(0xffffffffu, th, b0 + 3);
+        const int c0 = __shfl_sync(0xffffffffu, cnt, b0), c3 = __shfl_sync(0xffffffffu, cnt, b0 + 3);
+        const int e0 = __shfl_sync(0xffffffffu, ex, b0), e1 = __shfl_sync(0xffffffffu, ex, b0 + 1);
+        const int e2 = __shfl_sync(0xffffffffu, ex, b0 + 2), e3 = __shfl_sync(0xffffffffu, ex, b0 + 3);
+        if (c0 == target && c3 == target + 1 && e0 == e1 && e1 == e2 && e2 == e3 &&
+            x3 - x0 <= 0x1p-7 * x3) {
+          const int be = __shfl_sync(0xffffffffu, biased_exponent(det), fl);
+          const double v = det * pow2(be > 2045 ? -1022 : 1023 - be);
+          const double vi = __shfl_sync(0xffffffffu, v, b0 + q);
+          const double va = __shfl_sync(0xffffffffu, v, b0 + ((q + 1) & 3));
+          const double vb = __shfl_sync(0xffffffffu, v, b0 + ((q + 2) & 3));
+          const double vc = __shfl_sync(0xffffffffu, v, b0 + ((q + 3) & 3));
+          const double di = __shfl_sync(0xffffffffu, th, b0 + q) - lo;
+          double t = (di * va * vb * vc) / ((va - vi) * (vb - vi) * (vc - vi));
+          t += __shfl_xor_sync(0xffffffffu, t, 1);
+          t += __shfl_xor_sync(0xffffffffu, t, 2);
+          est = lo + t;
+          probe = est > lo && est < hi;  // the same in every lane (false for NaN)
+        }
+      }
     }
   }
   if (a.tstamp && pi.is_final && lane == 0) {  // multisection rounds (timing mode)
@@ -673,7 +777,7 @@ __global__ void __launch_bounds__(kWS * 32) k_sigma(ProjArgs a, ProjWork w) {
   if (lane == 0) {
     double wgt = (dv != 0.0) ? ldexp(-q / dv, eq - ev) : 0.0;
     if (!(wgt >= 0.0)) wgt = 0.0;
-    __stcg(S.sig + i, th);
+    __stcg(S.sig + i, th * unscale);
     __stcg(S.c2 + i, 2.0 * pi.beta * pi.beta * wgt);
   }
 }
@@ -696,10 +800,6 @@ constexpr int kWL = 4;           // warps per block
 constexpr int kMaxBisect = 160;  // rounds (the bracket needs ~13 + 52 at most)
 constexpr int kNewtonSteps = 4;
 
-__device__ __forceinline__ int biased_exponent(double x) {
-  return (int)((__double_as_longlong(x) >> 52) & 0x7ff);
-}
-
 // One bisection round of a lane (work = false: evaluate, keep the bracket,
 // so that the warp stays converged).  Trial point: 2^-16 hi while lo = 0;
 // lo 2^(d/2) while hi spans d >= 2 octaves above lo (exact scalings); else
@@ -714,7 +814,9 @@ __device__ __forceinline__ void bisect_round(const double* t2, int n, int k, int
     th = lo * __longlong_as_double((long long)(1023 + d / 2) << 52);
   else
     th = fma(0.5, hi - lo, lo);
-  const int cnt = sturm_count(t2, n, th) - (k + 1);
+  double det;
+  int ex;
+  const int cnt = sturm_count(t2, n, th, det, ex) - (k + 1);
   if (work) {
     if (cnt > target) {
       hi = th;
@@ -740,24 +842,8 @@ __global__ void __launch_bounds__(kWL * 32) k_sigma_lanes(ProjArgs a, ProjWork w
   double* bev = alv + K1;     // beta_1..beta_k at 1..k
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int n = 2 * k + 1;
-  unsigned long long mx = 0;
-  for (int q = tid; q < k; q += blockDim.x) {
-    const double al = ldg_cg(S.al + q), be = ldg_cg(S.be + q + 1);
-    alv[q] = al;
-    bev[q + 1] = be;
-    t2[2 * q + 1] = al * al;
-    t2[2 * q + 2] = be * be;
-    const unsigned long long ba = (unsigned long long)__double_as_longlong(al) & 0x7fffffffffffffffull;
-    const unsigned long long bb = (unsigned long long)__double_as_longlong(be) & 0x7fffffffffffffffull;
-    mx = max(mx, max(ba, bb));
-  }
-  if (tid == 0) t2[2 * k + 1] = 0.0;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  if (lane == 0) gmax[warp] = mx;
-  __syncthreads();
-  for (int q = 0; q < kWL; ++q) mx = max(mx, gmax[q]);
-  const double G = 2.0 * __longlong_as_double((long long)mx);
+  double unscale;
+  const double G = load_tridiagonal(S.al, S.be, k, t2, alv, bev, gmax, unscale);
   const int wbase = i0 + warp * 32;
   if (wbase > k) return;  // whole warp past the problem (warp-uniform)
   const int i = wbase + lane;
@@ -818,7 +904,7 @@ __global__ void __launch_bounds__(kWL * 32) k_sigma_lanes(ProjArgs a, ProjWork w
     minors(t2, n, th, true, q, dq, eq);
     double wgt = (dv != 0.0) ? ldexp(-q / dv, eq - ev) : 0.0;
     if (!(wgt >= 0.0)) wgt = 0.0;
-    __stcg(S.sig + i, th);
+    __stcg(S.sig + i, th * unscale);
     __stcg(S.c2 + i, 2.0 * pi.beta * pi.beta * wgt);
   }
   if (i == k) {  // null vector of B^T, as in k_sigma
@@ -849,9 +935,38 @@ __global__ void __launch_bounds__(kWL * 32) k_sigma_lanes(ProjArgs a, ProjWork w
 // residual and y (f_i = 1 for them, sigma_i c_i / (sigma_i^2 + lambda^2)
 // vanishes with sigma_i, and lambda = 0 drops them).  So where the sum misses
 // beta^2 by more than rounding (64 k eps beta^2), those c_i^2 share equally
-// what is left of beta^2.  One block per problem.
-__global__ void __launch_bounds__(kT) k_weights(ProjArgs a, ProjWork w) {
+// what is left of beta^2.  One block per problem; ngram further blocks per
+// final problem form the inner products of every group of kGroupQ right
+// reflectors for apply_q4, one warp per group.
+__global__ void __launch_bounds__(kT) k_weights(ProjArgs a, ProjWork w, int nprob, int ngram) {
   __shared__ double red[33];  // block_sum's scratch
+  if ((int)blockIdx.x >= nprob) {
+    const int x = blockIdx.x - nprob;
+    const ProbInfo pf = prob_info(a, a.nbatch > 1 ? x / ngram : nprob - 1);
+    const int k = pf.k, lane = threadIdx.x & 31;
+    const int g = (x % ngram) * (kT / 32) + (threadIdx.x >> 5), j0 = g * kGroupQ;
+    if (j0 >= k) return;
+    const Slots S = slot_of(w, pf);
+    double d[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    for (int c = j0 + lane; c < k; c += 32) {
+      double q[kGroupQ];
+#pragma unroll
+      for (int e = 0; e < kGroupQ; ++e)
+        q[e] = j0 + e < k && c >= j0 + e ? ldg_cg(S.Qs + (int64_t)(j0 + e) * k + c) : 0.0;
+      d[0] = fma(q[0], q[1], d[0]);
+      d[1] = fma(q[0], q[2], d[1]);
+      d[2] = fma(q[0], q[3], d[2]);
+      d[3] = fma(q[1], q[2], d[3]);
+      d[4] = fma(q[1], q[3], d[4]);
+      d[5] = fma(q[2], q[3], d[5]);
+    }
+#pragma unroll
+    for (int e = 0; e < 6; ++e) {
+      d[e] = warp_sum_d(d[e]);
+      if (lane == 0) __stcg(S.gram + 6 * g + e, d[e]);
+    }
+    return;
+  }
   const ProbInfo pi = prob_info(a, blockIdx.x);
   const int k = pi.k;
   if (k == 0) return;  // block-uniform
@@ -910,7 +1025,7 @@ __global__ void __launch_bounds__(kWB * 32) k_gcv_grid(ProjArgs a, ProjWork w) {
   if (!(s1 > 0.0)) return;
   const double mrows = a.mvec ? (double)a.mvec[pi.p] : (double)a.m;
   const double omega = a.rule == LSLU_LAMBDA_WGCV ? (double)(k + 1) / mrows : 1.0;
-  const double lam = s1 * pow(10.0, -14.0 + 0.0625 * t);
+  const double lam = grid_lambda(s1, t);
   const double L2 = lam * lam;
   double num = 0.0, den = 0.0;
   for (int i = lane; i < k; i += 32) {
@@ -981,6 +1096,162 @@ __device__ void apply_q(const Slots& S, int k, const double* z, double* yp,
   for (int e = 0; e < NP; ++e) {
     const int c = tid + kTF * e;
     if (c < k) yp[c] = zr[e];
+  }
+}
+
+// apply_q for k <= 4 kTF with kGroupQ reflectors at a time: their inner
+// products with z come out of one reduction, and what each takes off the
+// later ones' products follows from the reflectors' own inner products
+// (k_weights).  An FP64 instruction costs 64 cycles, so a reflector at a time
+// is bound by its reduction and barrier (about 1300 cycles at k = 50, 1500 at
+// 300); in groups it is ~550 and ~900.
+template <int NP>
+__device__ void apply_q4(const Slots& S, int k, const double* z, double* yp, double* red4,
+                         int& par) {
+  const int tid = threadIdx.x;
+  double zr[NP], qn[kGroupQ][NP], taun[kGroupQ], gn[6];
+  auto load = [&](int g) {
+#pragma unroll
+    for (int b = 0; b < kGroupQ; ++b) {
+      const int j = g * kGroupQ + b;
+      taun[b] = j < k ? ldg_cg(S.taur + j) : 0.0;
+#pragma unroll
+      for (int e = 0; e < NP; ++e) {
+        const int c = tid + kTF * e;
+        qn[b][e] = j < k && c < k && c >= j ? ldg_cg(S.Qs + (int64_t)j * k + c) : 0.0;
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 6; ++e) gn[e] = ldg_cg(S.gram + 6 * g + e);
+  };
+#pragma unroll
+  for (int e = 0; e < NP; ++e) zr[e] = tid + kTF * e < k ? z[tid + kTF * e] : 0.0;
+  int g = (k - 1) / kGroupQ;
+  load(g);
+  for (; g >= 0; --g) {
+    double q[kGroupQ][NP], t[kGroupQ], gm[6], u[kGroupQ];
+#pragma unroll
+    for (int b = 0; b < kGroupQ; ++b) {
+      t[b] = taun[b];
+      u[b] = 0.0;
+#pragma unroll
+      for (int e = 0; e < NP; ++e) {
+        q[b][e] = qn[b][e];
+        u[b] = fma(q[b][e], zr[e], u[b]);
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 6; ++e) gm[e] = gn[e];
+    if (g > 0) load(g - 1);
+    block_sum4(u, red4, par);
+    const double h3 = t[3] * u[3];
+    const double h2 = t[2] * fma(-h3, gm[5], u[2]);
+    const double h1 = t[1] * fma(-h2, gm[3], fma(-h3, gm[4], u[1]));
+    const double h0 = t[0] * fma(-h1, gm[0], fma(-h2, gm[1], fma(-h3, gm[2], u[0])));
+#pragma unroll
+    for (int e = 0; e < NP; ++e)
+      zr[e] = fma(-h0, q[0][e], fma(-h1, q[1][e], fma(-h2, q[2][e], fma(-h3, q[3][e], zr[e]))));
+  }
+#pragma unroll
+  for (int e = 0; e < NP; ++e)
+    if (tid + kTF * e < k) yp[tid + kTF * e] = zr[e];
+}
+
+// z = argmin ||beta e1 - B z||^2 + lambda^2 ||z||^2 by the Givens sweep for
+// damped bidiagonal least squares on B / sigma_1 (rotations do not depend on
+// the scale; the scaled entries cannot overflow when squared), by warp 0.
+//   q_j = rbar_j^2 + lambda^2 (the lambda row removed), rho_j^2 = q_j + beta_{j+1}^2,
+//   rbar_{j+1} = -alpha_{j+1} sqrt(q_j) / rho_j, phi_j = (rbar_j / rho_j) phibar_j,
+//   phibar_{j+1} = (beta_{j+1} / rho_j) (rbar_j / sqrt(q_j)) phibar_j,
+//   z_j = (phi_j - (beta_{j+1} alpha_{j+1} / rho_j) z_{j+1}) / rho_j.
+// rbar^2 follows a Moebius map with non-negative coefficients, so lane t
+// composes those of its ceil(k / 32) steps (2 x 2 matrices without
+// cancellation, rescaled on their exponent bits), a warp scan gives every
+// lane the rbar^2 its steps start from, and phibar is a prefix product; only
+// the back substitution, one FMA per step, stays sequential.  One thread
+// taking the sweep step by step needed about 1900 cycles per step (46 us at
+// k = 50, 278 at 300).  fac (k entries) is scratch; z ends in ph.
+__device__ void damped_sweep(const double* al, const double* be, int k, double beta, double s1,
+                             double lam, double* rinv, double* thv, double* ph, double* fac) {
+  const int lane = threadIdx.x & 31;
+  const double sc = s1 > 0.0 ? 1.0 / s1 : 1.0;
+  const double lm = lam * sc, L2 = lm * lm;
+  const int steps = (k + 31) / 32;
+  const int j0 = lane * steps, j1 = min(k, j0 + steps);
+  // [A B; C D] of this lane's steps, applied to rbar_{j0}^2
+  double A = 1.0, B = 0.0, C = 0.0, D = 1.0;
+  auto keep_range = [&]() {
+    const int e = max(max(biased_exponent(A), biased_exponent(B)),
+                      max(biased_exponent(C), biased_exponent(D)));
+    if (e > 1023 + 200 || e < 1023 - 200) {
+      const int sft = 1023 - e;
+      A = rescaled(A, sft); B = rescaled(B, sft);
+      C = rescaled(C, sft); D = rescaled(D, sft);
+    }
+  };
+  for (int j = j0; j < j1; ++j) {
+    const double an = j + 1 < k ? al[j + 1] * sc : 0.0, bj = be[j + 1] * sc;
+    const double a2 = an * an, d = fma(bj, bj, L2);
+    const double u = a2 * fma(L2, C, A), v = a2 * fma(L2, D, B);
+    C = fma(d, C, A);
+    D = fma(d, D, B);
+    A = u;
+    B = v;
+    keep_range();
+  }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {  // the steps of all lanes up to this one
+    const double Ap = __shfl_up_sync(0xffffffffu, A, o), Bp = __shfl_up_sync(0xffffffffu, B, o);
+    const double Cp = __shfl_up_sync(0xffffffffu, C, o), Dp = __shfl_up_sync(0xffffffffu, D, o);
+    if (lane >= o) {
+      const double An = fma(A, Ap, B * Cp), Bn = fma(A, Bp, B * Dp);
+      const double Cn = fma(C, Ap, D * Cp), Dn = fma(C, Bp, D * Dp);
+      A = An; B = Bn; C = Cn; D = Dn;
+      keep_range();
+    }
+  }
+  const double a0 = al[0] * sc, R0 = a0 * a0;
+  A = __shfl_up_sync(0xffffffffu, A, 1);
+  B = __shfl_up_sync(0xffffffffu, B, 1);
+  C = __shfl_up_sync(0xffffffffu, C, 1);
+  D = __shfl_up_sync(0xffffffffu, D, 1);
+  double rbar = a0;
+  if (lane > 0 && j0 < k)
+    rbar = -copysign(sqrt(fma(A, R0, B) / fma(C, R0, D)), al[j0]);
+  double F = 1.0;
+  for (int j = j0; j < j1; ++j) {
+    const double bj = be[j + 1] * sc, an = j + 1 < k ? al[j + 1] * sc : 0.0;
+    const double q = fma(rbar, rbar, L2);
+    const double ir = rsqrt(fma(bj, bj, q));
+    const double iq = q > 0.0 ? rsqrt(q) : 0.0;
+    const double sn = bj * ir;
+    const double f = q > 0.0 ? sn * (rbar * iq) : sn;
+    rinv[j] = ir;
+    thv[j] = sn * an;
+    ph[j] = rbar * ir;
+    fac[j] = f;
+    F *= f;
+    rbar = -(q * iq * ir) * an;
+  }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double Fp = __shfl_up_sync(0xffffffffu, F, o);
+    if (lane >= o) F *= Fp;
+  }
+  double phibar = __shfl_up_sync(0xffffffffu, F, 1);
+  phibar = beta * sc * (lane > 0 ? phibar : 1.0);
+  for (int j = j0; j < j1; ++j) {
+    ph[j] = ph[j] * phibar * rinv[j];
+    thv[j] = -thv[j] * rinv[j];
+    phibar *= fac[j];
+  }
+  __syncwarp();
+  if (lane == 0) {  // back substitution; z overwrites ph
+    double zj = ph[k - 1];
+    for (int j = k - 2; j >= 0; --j) {
+      zj = fma(thv[j], zj, ph[j]);
+      ph[j] = zj;
+    }
   }
 }
 
@@ -1064,12 +1335,12 @@ __global__ void __launch_bounds__(kTF) k_finish(ProjArgs a, ProjWork w) {
     __syncthreads();
     const int ib = ibest;
     const double gib = ldg_cg(S.gv + ib);
-    lam = s1 * pow(10.0, -14.0 + 0.0625 * ib);
+    lam = grid_lambda(s1, ib);
     if (ib > 0 && ib < kGrid - 1) {
       // bisection in log(lambda) between the neighbours: the midpoint of
       // log(lo) and log(hi) is log(sqrt(lo hi)), and mu = lambda^2 = lo hi
-      double lo = s1 * pow(10.0, -14.0 + 0.0625 * (ib - 1));
-      double hi = s1 * pow(10.0, -14.0 + 0.0625 * (ib + 1));
+      const double lo = grid_lambda(s1, ib - 1);
+      const double hi = grid_lambda(s1, ib + 1);
       auto slope = [&](double mu) {
         const GcvSums g = gcv_sums(sig2, c2, k, mu, omega, red4, par);
         return g.dN * g.D - 2.0 * g.N * g.dD;
@@ -1126,51 +1397,20 @@ __global__ void __launch_bounds__(kTF) k_finish(ProjArgs a, ProjWork w) {
   if (!(pi.is_final && a.want_y && yp)) return;
 
   if (ts) ts[5] = gtimer();
-  // ---- z = argmin ||beta e1 - B z||^2 + lambda^2 ||z||^2 ---------------------
-  // Givens sweep on B / sigma_1 (rotations do not depend on the scale; the
-  // scaled entries cannot overflow when squared), one thread.
-  if (tid == 0) {
-    const double sc = s1 > 0.0 ? 1.0 / s1 : 1.0;
-    const double lm = lam * sc;
-    const double L2 = lm * lm;
-    double rbar = al[0] * sc, phibar = beta * sc;
-    for (int j = 0; j < k; ++j) {
-      const double bj = be[j + 1] * sc;
-      const double q = fma(rbar, rbar, L2);  // r1^2 after removing lambda-row j
-      const double ir = rsqrt(fma(bj, bj, q));  // 1 / r after removing beta_{j+1}
-      double c1 = 1.0, r1 = rbar;  // lambda = 0: no first rotation
-      if (lm != 0.0) {
-        const double iq = rsqrt(q);
-        c1 = rbar * iq;
-        r1 = q * iq;
-      }
-      const double cs = r1 * ir, sn = bj * ir;
-      const double phib = c1 * phibar;
-      rinv[j] = ir;
-      ph[j] = cs * phib;
-      phibar = sn * phib;
-      if (j + 1 < k) {
-        const double an = al[j + 1] * sc;
-        thv[j] = sn * an;
-        rbar = -cs * an;
-      }
-    }
-    // back substitution; z overwrites ph
-    ph[k - 1] *= rinv[k - 1];
-    for (int j = k - 2; j >= 0; --j) ph[j] = (ph[j] - thv[j] * ph[j + 1]) * rinv[j];
-  }
+  __syncthreads();  // sig2 and c2 have been read; sig2 is scratch below
+  if (warp == 0) damped_sweep(al, be, k, beta, s1, lam, rinv, thv, ph, sig2);
   __syncthreads();
   if (ts) ts[6] = gtimer();
   // ---- y = Q z ----------------------------------------------------------------
   const int np = (k + kTF - 1) / kTF;
   if (np <= 1)
-    apply_q<1>(S, k, ph, yp, qred);
+    apply_q4<1>(S, k, ph, yp, red4, par);
   else if (np <= 2)
-    apply_q<2>(S, k, ph, yp, qred);
+    apply_q4<2>(S, k, ph, yp, red4, par);
   else if (np <= 3)
-    apply_q<3>(S, k, ph, yp, qred);
+    apply_q4<3>(S, k, ph, yp, red4, par);
   else if (np <= 4)
-    apply_q<4>(S, k, ph, yp, qred);
+    apply_q4<4>(S, k, ph, yp, red4, par);
   else if (np <= 8)
     apply_q<8>(S, k, ph, yp, qred);
   else
@@ -1246,7 +1486,7 @@ __global__ void __launch_bounds__(kT) k_opt_grid(ProjWork w, int K, const DevSta
     if (threadIdx.x == 0) Eg[blockIdx.x] = 0.0;
     return;
   }
-  const double lam = s1 * pow(10.0, -14.0 + 0.0625 * (int)blockIdx.x);
+  const double lam = grid_lambda(s1, (int)blockIdx.x);
   const double e = opt_eval(S, k, st->beta, lam, G, g, sm, red);
   if (threadIdx.x == 0) Eg[blockIdx.x] = e;
 }
@@ -1273,11 +1513,11 @@ __device__ bool opt_bracket(int r, double s1, const double* Eg, const double* Er
   for (int i = 1; i < kGrid; ++i)
     if (Eg[i] < Eg[b]) b = i;
   if (b == 0 || b == kGrid - 1) {
-    lo = hi = log(s1 * pow(10.0, -14.0 + 0.0625 * b));
+    lo = hi = log(grid_lambda(s1, b));
     return false;
   }
-  lo = log(s1 * pow(10.0, -14.0 + 0.0625 * (b - 1)));
-  hi = log(s1 * pow(10.0, -14.0 + 0.0625 * (b + 1)));
+  lo = log(grid_lambda(s1, b - 1));
+  hi = log(grid_lambda(s1, b + 1));
   for (int q = 0; q < r; ++q) {
     const double h = (hi - lo) / (kOptPts + 1);
     int j = 0;
@@ -1337,7 +1577,7 @@ __global__ void k_opt_pick(ProjWork w, int K, const DevState* st, const double* 
 }  // namespace
 
 int64_t projected_slot_doubles(int kk, int /*CL*/) {
-  return 5 * (int64_t)(kk + 1) + kGrid + 1 + (int64_t)kk * kk + (int64_t)(kk + 1) * kk + 64;
+  return 5 * (int64_t)(kk + 1) + kGrid + 1 + gram_doubles(kk) + (int64_t)kk * kk + (int64_t)(kk + 1) * kk + 64;
 }
 
 // Per-device set-up of the projected kernels: their attributes (cluster size
@@ -1469,7 +1709,9 @@ cudaError_t launch_projected(const ProjArgs& a, ProjWork& w, cudaStream_t s, int
     k_sigma<<<g2, kWS * 32, sm2, s>>>(a, w);
     w.prob0 = 0;
   }
-  k_weights<<<(unsigned)nprob, kT, 0, s>>>(a, w);
+  const int groups = (kmax + kGroupQ - 1) / kGroupQ;
+  const int ngram = a.want_y ? (groups + kT / 32 - 1) / (kT / 32) : 0;
+  k_weights<<<(unsigned)(nprob + ngram * (batch ? nprob : 1)), kT, 0, s>>>(a, w, nprob, ngram);
   // 3. the GCV function on the lambda grid
   const bool grid = a.rule == LSLU_LAMBDA_GCV || a.rule == LSLU_LAMBDA_WGCV;
   if (grid) {
