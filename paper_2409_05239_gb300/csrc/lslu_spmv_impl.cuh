@@ -389,6 +389,13 @@ __device__ __forceinline__ YT row_dot(const RowAt& r, const ColIdx ci, const VT*
     return row_dot_len<VT, XT, YT, G, U>(r.start, r.len, ci.col, val, x, gl);
 }
 
+// The shapes whose blocks take several row groups (the default FP32 / BF16
+// products); the others have one group per block.
+template <int G, int U>
+__host__ __device__ constexpr bool takes_several_groups() {
+  return G != 0 && U >= 4;
+}
+
 // The rows of block b of nb (row groups b, b + nb, ... of 256 / GL rows): y =
 // A x on them, with the next group's row pointers read ahead.
 template <typename VT, typename XT, typename YT, int G, int U, int F>
@@ -407,8 +414,8 @@ __device__ __forceinline__ void stream_rows(int64_t b, int64_t nb, int64_t rows,
   RowAt r = row_at<F>(row, row < rows, rp, rl, ci);
   while (true) {
     const int64_t next = row + stride;
-    // (the same for the whole warp; the other shapes have one group per block)
-    const bool more = U >= 4 && G != 0 && next - in_warp < rows;
+    // the same for the whole warp
+    const bool more = takes_several_groups<G, U>() && next - in_warp < rows;
     RowAt rn = {0, 0, 0};
     if (more) rn = row_at<F>(next, next < rows, rp, rl, ci);
     const YT acc = row_dot<VT, XT, YT, G, U, F>(r, ci, val, x, gl);
@@ -549,9 +556,9 @@ inline ColIdx col_idx(const DevCsr& A) { return {A.col, A.off, A.ubase, A.bbase,
 // the pivot blocks, each taking several groups.  Where the pivot blocks of a
 // batch alone fill half the GPU, blocks of two groups instead: resident blocks
 // of equal shares would wait for the ones that start late.
-template <int U>
+template <int G, int U>
 int64_t stream_blocks(const DevCsr& A, int64_t groups, int64_t npiv) {
-  if (U < 4 || A.num_sms <= 0) return groups;
+  if (!takes_several_groups<G, U>() || A.num_sms <= 0) return groups;
   const int64_t slots = (int64_t)A.num_sms * kStreamBlocksPerSm;
   const int64_t nb = npiv <= slots / 2 ? slots - npiv : (groups + 1) / 2;
   return groups < nb ? groups : nb;
@@ -561,7 +568,7 @@ template <typename VT, typename XT, typename YT, int G, int U, bool DEF = false>
 void spmv_run(const DevCsr& A, const XT* x, YT* y, cudaStream_t s) {
   if (A.rows == 0) return;
   constexpr int RPB = 256 / (G == 0 ? 32 : G);
-  const int64_t blocks = stream_blocks<U>(A, (A.rows + RPB - 1) / RPB, 0);
+  const int64_t blocks = stream_blocks<G, U>(A, (A.rows + RPB - 1) / RPB, 0);
   const VT* v = reinterpret_cast<const VT*>(A.val);
   with_format<DEF>(A, [&](auto F) {
     k_spmv<VT, XT, YT, G, U, F.value><<<(unsigned)blocks, 256, 0, s>>>(
@@ -573,7 +580,7 @@ template <typename VT, typename XT, typename YT, int G, int U, bool DEF = false>
 void spmv_pivots_run(const DevCsr& A, const XT* x, YT* y, const PivotCoef& pc, cudaStream_t s) {
   constexpr int RPB = 256 / (G == 0 ? 32 : G);
   const int64_t npiv = (int64_t)pc.npiv_blocks * pc.nprob;
-  const int64_t blocks = npiv + stream_blocks<U>(A, (A.rows + RPB - 1) / RPB, npiv);
+  const int64_t blocks = npiv + stream_blocks<G, U>(A, (A.rows + RPB - 1) / RPB, npiv);
   const VT* v = reinterpret_cast<const VT*>(A.val);
   with_format<DEF>(A, [&](auto F) {
     launch_pdl(k_spmv_pivots<VT, XT, YT, G, U, F.value>, dim3((unsigned)blocks), dim3(256), 0, s,
