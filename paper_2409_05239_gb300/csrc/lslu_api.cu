@@ -107,7 +107,9 @@ namespace {
 // Device state of a handle whose padded concatenated CSR (c->m x c->n rows,
 // c->nprob problems) is rp/ci/vv; every per-problem array is strided.
 lslu_status create_common(lslu_ctx* c, const int64_t* rp, const int32_t* ci, const double* vv,
-                          int64_t csr_m = -1, int64_t csr_n = -1) {
+                          int64_t csr_m = -1, int64_t csr_n = -1, bool on_device = false,
+                          const std::vector<int32_t>* inv_row = nullptr,
+                          const std::vector<int32_t>* col_new = nullptr) {
   lslu_status st = LSLU_OK;
   auto fail = [&](lslu_status s2) {
     lslu::thread_error() = c->err;
@@ -127,8 +129,8 @@ lslu_status create_common(lslu_ctx* c, const int64_t* rp, const int32_t* ci, con
   const int P = c->nprob;
   CKC(cudaGetDevice(&c->device));
   CKC(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device));
-  CKC(build_csr_pair(csr_m < 0 ? m : csr_m, csr_n < 0 ? n : csr_n, rp, ci, vv, c->value_type,
-                     &c->A, &c->AT, c->stream));
+  CKC(build_csr_pair(csr_m < 0 ? m : csr_m, csr_n < 0 ? n : csr_n, rp, ci, vv, on_device, inv_row,
+                     col_new, c->value_type, &c->A, &c->AT, c->stream));
   if (c->shared_rhs)
     CKC(dmalloc(&c->xi, (size_t)std::max(c->m1, c->n1) * rhs_stride(c->shared_rhs)));
   const int K = c->kmax;
@@ -234,27 +236,26 @@ lslu_status read_order(const int32_t* order, int64_t len, bool device, std::vect
   return LSLU_OK;
 }
 
-// A host CSR renumbered: stored row r holds caller row inv_row[r], with its
-// columns mapped through col_new and sorted ascending (stable for repeats).
-void renumber_csr(int64_t rows, const int64_t* rp, const int32_t* ci, const double* vv,
-                  const std::vector<int32_t>& inv_row, const std::vector<int32_t>& col_new,
-                  std::vector<int64_t>& rp_o, std::vector<int32_t>& ci_o,
-                  std::vector<double>& vv_o) {
-  rp_o.assign(rows + 1, 0);
-  for (int64_t r = 0; r < rows; ++r)
-    rp_o[r + 1] = rp_o[r] + (rp[inv_row[r] + 1] - rp[inv_row[r]]);
-  ci_o.resize(rp_o[rows]);
-  vv_o.resize(rp_o[rows]);
-  std::vector<uint64_t> key;
-  for (int64_t r = 0; r < rows; ++r) {
-    const int64_t a = rp[inv_row[r]], len = rp[inv_row[r] + 1] - a, o = rp_o[r];
-    key.resize(len);
-    for (int64_t i = 0; i < len; ++i)
-      key[i] = ((uint64_t)(uint32_t)col_new[ci[a + i]] << 32) | (uint64_t)i;
-    std::sort(key.begin(), key.end());
-    for (int64_t i = 0; i < len; ++i) {
-      ci_o[o + i] = (int32_t)(key[i] >> 32);
-      vv_o[o + i] = vv[a + (int64_t)(key[i] & 0xffffffffull)];
+// First entry with a column outside [0, n) and first non-finite value (-1:
+// none).  Branch-free passes over chunks, so that the compiler vectorises them.
+void check_csr_host(int64_t nnz, int64_t n, const int32_t* ci, const double* vv, int64_t* bad_col,
+                    int64_t* bad_val) {
+  *bad_col = *bad_val = -1;
+  const uint32_t lim = (uint32_t)std::min<int64_t>(n, INT32_MAX);
+  constexpr int64_t kChunk = 4096;
+  for (int64_t a = 0; a < nnz && *bad_col < 0 && *bad_val < 0; a += kChunk) {
+    const int64_t b = std::min(nnz, a + kChunk);
+    uint32_t cbad = 0;
+    uint64_t vbad = 0;
+    for (int64_t i = a; i < b; ++i) cbad |= (uint32_t)((uint32_t)ci[i] >= lim);
+    for (int64_t i = a; i < b; ++i) {
+      uint64_t u;
+      std::memcpy(&u, vv + i, 8);
+      vbad |= (uint64_t)((u & 0x7ff0000000000000ull) == 0x7ff0000000000000ull);
+    }
+    for (int64_t i = a; i < b && (cbad || vbad); ++i) {
+      if (*bad_col < 0 && (uint32_t)ci[i] >= lim) *bad_col = i;
+      if (*bad_val < 0 && !std::isfinite(vv[i])) *bad_val = i;
     }
   }
 }
@@ -279,35 +280,34 @@ lslu_status create_single(int64_t m, int64_t n, int64_t nnz, const int64_t* row_
   if (!row_ptr || (nnz > 0 && (!col_idx || !vals)))
     return set_err(nullptr, LSLU_ERR_INVALID_ARG, "NULL CSR array");
 
-  // bring the CSR to the host for validation and layout
-  std::vector<int64_t> rp(m + 1);
-  std::vector<int32_t> ci(nnz);
-  std::vector<double> vv(nnz);
-  if (ptr_location == LSLU_DEVICE) {
-    cudaError_t e = cudaMemcpy(rp.data(), row_ptr, (m + 1) * 8, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess && nnz)
-      e = cudaMemcpy(ci.data(), col_idx, nnz * 4, cudaMemcpyDeviceToHost);
-    if (e == cudaSuccess && nnz) e = cudaMemcpy(vv.data(), vals, nnz * 8, cudaMemcpyDeviceToHost);
+  // row pointers on the host; columns and values stay where they are
+  const bool on_device = ptr_location == LSLU_DEVICE;
+  std::vector<int64_t> rp_h;
+  if (on_device) {
+    rp_h.resize(m + 1);
+    const cudaError_t e = cudaMemcpy(rp_h.data(), row_ptr, (m + 1) * 8, cudaMemcpyDeviceToHost);
     if (e != cudaSuccess)
       return set_err(nullptr, LSLU_ERR_CUDA, std::string("copying CSR: ") + cudaGetErrorString(e));
-  } else {
-    std::memcpy(rp.data(), row_ptr, (m + 1) * 8);
-    if (nnz) {
-      std::memcpy(ci.data(), col_idx, nnz * 4);
-      std::memcpy(vv.data(), vals, nnz * 8);
-    }
+    row_ptr = rp_h.data();
   }
-  if (rp[0] != 0 || rp[m] != nnz)
+  if (row_ptr[0] != 0 || row_ptr[m] != nnz)
     return set_err(nullptr, LSLU_ERR_INVALID_ARG, "row_ptr[0] must be 0 and row_ptr[m] == nnz");
   for (int64_t r = 0; r < m; ++r)
-    if (rp[r + 1] < rp[r])
+    if (row_ptr[r + 1] < row_ptr[r])
       return set_err(nullptr, LSLU_ERR_INVALID_ARG, "row_ptr is not monotone");
-  for (int64_t i = 0; i < nnz; ++i) {
-    if (ci[i] < 0 || ci[i] >= n)
-      return set_err(nullptr, LSLU_ERR_INVALID_ARG, "column index out of range");
-    if (!std::isfinite(vv[i]))
-      return set_err(nullptr, LSLU_ERR_INVALID_ARG, "non-finite matrix value");
+  int64_t bad_col = -1, bad_val = -1;
+  if (on_device) {
+    const cudaError_t e = check_csr_device(nnz, n, col_idx, vals, (cudaStream_t)cuda_stream,
+                                           &bad_col, &bad_val);
+    if (e != cudaSuccess)
+      return set_err(nullptr, e == cudaErrorMemoryAllocation ? LSLU_ERR_OOM : LSLU_ERR_CUDA,
+                     std::string("checking CSR: ") + cudaGetErrorString(e));
+  } else {
+    check_csr_host(nnz, n, col_idx, vals, &bad_col, &bad_val);
   }
+  if (bad_col >= 0 && (bad_val < 0 || bad_col <= bad_val))
+    return set_err(nullptr, LSLU_ERR_INVALID_ARG, "column index out of range");
+  if (bad_val >= 0) return set_err(nullptr, LSLU_ERR_INVALID_ARG, "non-finite matrix value");
   const bool ordered = row_order || col_order;
   std::vector<int32_t> om, on, im, in;
   if (ordered) {
@@ -315,13 +315,6 @@ lslu_status create_single(int64_t m, int64_t n, int64_t nnz, const int64_t* row_
     if (st == LSLU_OK)
       st = read_order(col_order, n, ptr_location == LSLU_DEVICE, on, in, "col_order");
     if (st != LSLU_OK) return st;
-    std::vector<int64_t> rp2;
-    std::vector<int32_t> ci2;
-    std::vector<double> vv2;
-    renumber_csr(m, rp.data(), ci.data(), vv.data(), im, on, rp2, ci2, vv2);
-    rp.swap(rp2);
-    ci.swap(ci2);
-    vv.swap(vv2);
   }
 
   c = new lslu_ctx();
@@ -338,7 +331,8 @@ lslu_status create_single(int64_t m, int64_t n, int64_t nnz, const int64_t* row_
   c->value_type = value_type;
   c->kmax = max_iter;
   c->stream = (cudaStream_t)cuda_stream;
-  lslu_status st = create_common(c, rp.data(), ci.data(), vv.data());
+  lslu_status st = create_common(c, row_ptr, col_idx, vals, -1, -1, on_device,
+                                 ordered ? &im : nullptr, ordered ? &on : nullptr);
   if (st != LSLU_OK) return st;
   if (ordered) {
     cudaError_t e = dmalloc(&c->ord_m, m);

@@ -373,9 +373,22 @@ inline void launch_spmv_pivots_shape(int shape, const DevCsr& A, int vt, const v
     launch_spmv_pivots_shape_b(g, A, vt, x, y, pc, s);
 }
 
-// Build the padded CSR of A and of A^T (host-side layout, then upload).
+// The stored matrices of a handle (lslu_build.cu) from a validated CSR: rp on
+// the host, ci and vv on the host or (on_device) the device; inv_row and
+// col_new (both or neither) renumber it (stored row r is caller row inv_row[r],
+// columns mapped through col_new and sorted).  check_csr_device: first entry
+// with a column outside [0, n) and first non-finite value of a device CSR, -1
+// where there is none.
 cudaError_t build_csr_pair(int64_t m, int64_t n, const int64_t* rp, const int32_t* ci,
-                           const double* vv, int vt, DevCsr* A, DevCsr* AT, cudaStream_t s);
+                           const double* vv, bool on_device, const std::vector<int32_t>* inv_row,
+                           const std::vector<int32_t>* col_new, int vt, DevCsr* A, DevCsr* AT,
+                           cudaStream_t s);
+cudaError_t check_csr_device(int64_t nnz, int64_t n, const int32_t* ci, const double* vv,
+                             cudaStream_t s, int64_t* bad_col, int64_t* bad_val);
+void renumber_csr(int64_t rows, const int64_t* rp, const int32_t* ci, const double* vv,
+                  const std::vector<int32_t>& inv_row, const std::vector<int32_t>& col_new,
+                  std::vector<int64_t>& rp_o, std::vector<int32_t>& ci_o,
+                  std::vector<double>& vv_o);
 void free_csr(DevCsr* c);
 
 // Basis-step kernels; see lslu_basis.cu.  Problem p's arrays sit at

@@ -174,220 +174,7 @@ __global__ void k_interleave(const float* __restrict__ x, int64_t xstride, int64
   }
 }
 
-uint16_t f32_to_bf16_rne(float f) {
-  uint32_t u;
-  std::memcpy(&u, &f, 4);
-  const uint32_t lsb = (u >> 16) & 1u;
-  return (uint16_t)((u + 0x7fffu + lsb) >> 16);
-}
-
-// Host-side construction of the padded CSR (values converted to the storage
-// type): rows start on multiples of kRowAlign; pad entries repeat the last
-// column of their row with value 0.
-cudaError_t upload_padded(int64_t rows, int64_t cols, const std::vector<int64_t>& rp,
-                          const std::vector<int32_t>& ci, const std::vector<double>& vv, int vt,
-                          DevCsr* out, cudaStream_t s) {
-  std::vector<int32_t> prp(rows + 1), prl(rows);
-  int64_t tot = 0;
-  for (int64_t r = 0; r < rows; ++r) {
-    const int64_t len = rp[r + 1] - rp[r];
-    const int64_t plen = (len + kRowAlign - 1) / kRowAlign * kRowAlign;
-    prp[r] = (int32_t)tot;
-    prl[r] = (int32_t)plen;
-    tot += plen;
-    if (tot >= (int64_t)INT32_MAX) return cudaErrorInvalidValue;
-  }
-  prp[rows] = (int32_t)tot;
-  std::vector<int32_t> pc((size_t)tot);
-  std::vector<double> pv((size_t)tot);
-  for (int64_t r = 0; r < rows; ++r) {
-    const int64_t a = rp[r], len = rp[r + 1] - rp[r];
-    int32_t* dc = pc.data() + prp[r];
-    double* dv = pv.data() + prp[r];
-    for (int64_t e = 0; e < len; ++e) {
-      dc[e] = ci[a + e];
-      dv[e] = vv[a + e];
-    }
-    for (int64_t e = len; e < prl[r]; ++e) {
-      dc[e] = len ? ci[a + len - 1] : 0;
-      dv[e] = 0.0;
-    }
-    // full kPermBlock-entry blocks stored transposed (4 x 16): position 4 l + i
-    // holds entry 16 i + l, so that the 16 lanes of a row group gather 16
-    // consecutive entries of the row in each step; the last partial block
-    // keeps its order
-    const int64_t nfull = prl[r] / kPermBlock;
-    for (int64_t b = 0; b < nfull; ++b) {
-      int32_t tc[kPermBlock];
-      double tv[kPermBlock];
-      const int64_t base = b * kPermBlock;
-      for (int l = 0; l < 16; ++l)
-        for (int i = 0; i < 4; ++i) {
-          tc[4 * l + i] = dc[base + 16 * i + l];
-          tv[4 * l + i] = dv[base + 16 * i + l];
-        }
-      for (int q = 0; q < kPermBlock; ++q) {
-        dc[base + q] = tc[q];
-        dv[base + q] = tv[q];
-      }
-    }
-  }
-  out->rows = rows;
-  out->cols = cols;
-  out->nnz = rp[rows];
-  out->nnz_padded = tot;
-  size_t vbytes = vt == LSLU_F64 ? 8 : (vt == LSLU_F32 ? 4 : 2);
-  cudaError_t e;
-  // row pointers padded to a multiple of 4 entries
-  const int64_t nrp = (rows + 1 + 3) / 4 * 4;
-  prp.resize((size_t)nrp, (int32_t)tot);
-  if ((e = cudaMalloc(&out->row_ptr, nrp * sizeof(int32_t))) != cudaSuccess) return e;
-  if ((e = cudaMalloc(&out->row_len, std::max<int64_t>(rows, 1) * sizeof(int32_t))) != cudaSuccess)
-    return e;
-  if ((e = cudaMalloc(&out->col, std::max<int64_t>(tot, kRowAlign) * sizeof(int32_t))) !=
-      cudaSuccess)
-    return e;
-  if ((e = cudaMalloc(&out->val, std::max<int64_t>(tot, kRowAlign) * vbytes)) != cudaSuccess)
-    return e;
-  if ((e = cudaMemcpyAsync(out->row_ptr, prp.data(), nrp * sizeof(int32_t),
-                           cudaMemcpyHostToDevice, s)) != cudaSuccess)
-    return e;
-  if (rows && (e = cudaMemcpyAsync(out->row_len, prl.data(), rows * sizeof(int32_t),
-                                   cudaMemcpyHostToDevice, s)) != cudaSuccess)
-    return e;
-  if (tot && (e = cudaMemcpyAsync(out->col, pc.data(), tot * sizeof(int32_t),
-                                  cudaMemcpyHostToDevice, s)) != cudaSuccess)
-    return e;
-  // 16-bit column offsets, from the smallest column of every 64-entry block of
-  // a row when each block spans fewer than 2^16 columns, else from that of
-  // every 8-entry unit (rows start and end on unit boundaries) when those do
-  const int64_t units = tot / kRowAlign;
-  std::vector<uint16_t> po;
-  std::vector<int32_t> pb, bb, rb;
-  auto span = [&](int64_t a, int64_t b, int32_t& lo) {
-    int32_t hi = lo = pc[a];
-    for (int64_t q = a + 1; q < b; ++q) {
-      lo = std::min(lo, pc[q]);
-      hi = std::max(hi, pc[q]);
-    }
-    return (int64_t)hi - lo <= 65535;
-  };
-  auto fill = [&](int64_t a, int64_t b, int32_t lo) {
-    for (int64_t q = a; q < b; ++q) po[q] = (uint16_t)(pc[q] - lo);
-    for (int64_t u = a / kRowAlign; u < b / kRowAlign; ++u) pb[u] = lo;
-  };
-  bool fits = units > 0, blocks_fit = units > 0;
-  if (fits) {
-    po.resize((size_t)tot);
-    pb.resize((size_t)units);
-    rb.resize((size_t)rows);
-    for (int64_t r = 0; r < rows && blocks_fit; ++r) {
-      rb[r] = (int32_t)bb.size();
-      for (int64_t a = prp[r]; a < prp[r] + prl[r] && blocks_fit; a += kPermBlock) {
-        const int64_t b = std::min<int64_t>(a + kPermBlock, prp[r] + prl[r]);
-        int32_t lo;
-        blocks_fit = span(a, b, lo);
-        if (blocks_fit) {
-          fill(a, b, lo);
-          bb.push_back(lo);
-        }
-      }
-    }
-    for (int64_t u = 0; u < units && fits && !blocks_fit; ++u) {
-      int32_t lo;
-      fits = span(u * kRowAlign, (u + 1) * kRowAlign, lo);
-      if (fits) fill(u * kRowAlign, (u + 1) * kRowAlign, lo);
-    }
-  }
-  if (fits) {
-    // unit bases readable up to a multiple of 4 units (aligned bulk copies)
-    const int64_t nub = (units + 3) / 4 * 4;
-    pb.resize((size_t)nub, 0);
-    if ((e = cudaMalloc(&out->off, tot * sizeof(uint16_t))) != cudaSuccess) return e;
-    if ((e = cudaMalloc(&out->ubase, nub * sizeof(int32_t))) != cudaSuccess) return e;
-    if ((e = cudaMemcpyAsync(out->off, po.data(), tot * sizeof(uint16_t), cudaMemcpyHostToDevice,
-                             s)) != cudaSuccess)
-      return e;
-    if ((e = cudaMemcpyAsync(out->ubase, pb.data(), nub * sizeof(int32_t),
-                             cudaMemcpyHostToDevice, s)) != cudaSuccess)
-      return e;
-    if (blocks_fit) {
-      if ((e = cudaMalloc(&out->bbase, bb.size() * sizeof(int32_t))) != cudaSuccess) return e;
-      if ((e = cudaMalloc(&out->rblk, rows * sizeof(int32_t))) != cudaSuccess) return e;
-      if ((e = cudaMemcpyAsync(out->bbase, bb.data(), bb.size() * sizeof(int32_t),
-                               cudaMemcpyHostToDevice, s)) != cudaSuccess)
-        return e;
-      if ((e = cudaMemcpyAsync(out->rblk, rb.data(), rows * sizeof(int32_t),
-                               cudaMemcpyHostToDevice, s)) != cudaSuccess)
-        return e;
-    }
-    if ((e = cudaStreamSynchronize(s)) != cudaSuccess) return e;  // po, pb.. go out of scope
-    out->compressed = 1;
-    out->block_compressed = blocks_fit;
-  }
-  if (tot) {
-    if (vt == LSLU_F64) {
-      e = cudaMemcpyAsync(out->val, pv.data(), tot * 8, cudaMemcpyHostToDevice, s);
-    } else if (vt == LSLU_F32) {
-      std::vector<float> f((size_t)tot);
-      for (int64_t i = 0; i < tot; ++i) f[i] = (float)pv[i];
-      e = cudaMemcpyAsync(out->val, f.data(), tot * 4, cudaMemcpyHostToDevice, s);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    } else {
-      std::vector<uint16_t> h((size_t)tot);
-      for (int64_t i = 0; i < tot; ++i) h[i] = f32_to_bf16_rne((float)pv[i]);
-      e = cudaMemcpyAsync(out->val, h.data(), tot * 2, cudaMemcpyHostToDevice, s);
-      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    }
-    if (e != cudaSuccess) return e;
-  }
-  return cudaStreamSynchronize(s);
-}
-
 }  // namespace
-
-cudaError_t build_csr_pair(int64_t m, int64_t n, const int64_t* rp, const int32_t* ci,
-                           const double* vv, int vt, DevCsr* A, DevCsr* AT, cudaStream_t s) {
-  const int64_t nnz = rp[m];
-  std::vector<int64_t> rpa(rp, rp + m + 1);
-  std::vector<int32_t> cia(ci, ci + nnz);
-  std::vector<double> va(vv, vv + nnz);
-  cudaError_t e = upload_padded(m, n, rpa, cia, va, vt, A, s);
-  if (e != cudaSuccess) return e;
-  // stable counting sort by column: rows of A^T list the rows of A in
-  // increasing order (entries of one row of A keep their input order)
-  std::vector<int64_t> rpt(n + 1, 0);
-  for (int64_t i = 0; i < nnz; ++i) rpt[cia[i] + 1]++;
-  for (int64_t c = 0; c < n; ++c) rpt[c + 1] += rpt[c];
-  std::vector<int64_t> cur(rpt.begin(), rpt.end() - 1);
-  std::vector<int32_t> cit((size_t)nnz);
-  std::vector<double> vt_((size_t)nnz);
-  for (int64_t r = 0; r < m; ++r)
-    for (int64_t i = rpa[r]; i < rpa[r + 1]; ++i) {
-      const int64_t pos = cur[cia[i]]++;
-      cit[pos] = (int32_t)r;
-      vt_[pos] = va[i];
-    }
-  const cudaError_t e2 = upload_padded(n, m, rpt, cit, vt_, vt, AT, s);
-  A->shape = AT->shape = default_shape(vt);
-  int dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess)
-    cudaDeviceGetAttribute(&A->num_sms, cudaDevAttrMultiProcessorCount, dev);
-  AT->num_sms = A->num_sms;
-  return e2;
-}
-
-void free_csr(DevCsr* c) {
-  cudaFree(c->row_ptr);
-  cudaFree(c->row_len);
-  cudaFree(c->col);
-  cudaFree(c->val);
-  cudaFree(c->off);
-  cudaFree(c->ubase);
-  cudaFree(c->bbase);
-  cudaFree(c->rblk);
-  *c = DevCsr();
-}
 
 // 16 lanes per row with 8 entries in flight per lane (two 4-entry chunks of
 // 32-bit columns); FP64 values keep 4 in flight (registers).
