@@ -19,7 +19,6 @@ namespace lslu {
 namespace {
 
 constexpr int kGroup = 16;  // lanes per row of the shared-matrix product
-constexpr int kRowsPerBlock = 256 / kGroup;
 
 // ---- several right-hand sides sharing one matrix ---------------------------
 // The R input vectors are first interleaved, xi[j * RS + r] (RS = R rounded
@@ -92,27 +91,29 @@ __device__ __forceinline__ float row_dot_rhs(int64_t row, const int32_t* __restr
   return group_sum<kGroup>(acc);
 }
 
-template <int RS>
-__device__ __forceinline__ void gather_rhs(const float* __restrict__ xi, int32_t c, float (&xv)[RS]) {
-  const float4* p = reinterpret_cast<const float4*>(xi + (int64_t)c * RS);
-#pragma unroll
-  for (int q = 0; q < RS / 4; ++q) {
-    const float4 t = __ldg(p + q);
-    xv[4 * q] = t.x; xv[4 * q + 1] = t.y; xv[4 * q + 2] = t.z; xv[4 * q + 3] = t.w;
-  }
-}
-
 // y[r * ystride + row] = (A xi_r)(row) for r < R, rows of the shared CSR;
 // pivot blocks as in k_spmv_pivots, with output rows of problem p at
 // p * ystride + row.
+// RS / 4 threads stand for one lane of the single-vector group, each with four
+// right-hand sides, so a gather request reads whole 4 RS-byte rows of xi (one
+// thread gathering all of them took RS / 4 requests of 32 scattered 16-byte
+// pieces, and the L1's tag lookups bounded the product).  A warp takes one row
+// with RS = 16 (two of the 16 lanes per thread group, kept as separate
+// accumulators) or RS = 8, and two rows with RS = 4; the sums and the butterfly
+// are those of the 16 lanes, so every output keeps its bits.
+// 256x256 CT, 16 right-hand sides, K = 50: 163 -> 77 us per product, the solve
+// 21.0 -> 12.4 ms (all gathers of a step ahead of its sums: 12.8 to 13.8 ms).
 template <typename VT, int RS, int F>
-__global__ void __launch_bounds__(256, 4)
+__global__ void __launch_bounds__(256)
     k_spmm_pivots(int64_t rows, const int32_t* __restrict__ rp, const int32_t* __restrict__ rl,
                   const ColIdx ci, const VT* __restrict__ val, const float* __restrict__ xi,
                   float* __restrict__ y, int64_t ystride, int R, PivotCoef pc) {
   constexpr int C = kFmtChunk<F>;
   constexpr int S = kGroup * C;
-  const int lane = threadIdx.x & 31;
+  constexpr int T = RS / 4;                     // threads of one lane
+  constexpr int V = T == 4 ? 2 : 1;             // lanes per thread
+  constexpr int TEAM = kGroup / V * T;          // threads of one row
+  constexpr int RPB = 256 / TEAM;               // rows of a block
   const int npiv_all = pc.npiv_blocks * pc.nprob;
   if ((int)blockIdx.x < npiv_all) {
     pivot_blocks<float, kGroup>(pc, [=](int p, int32_t row, int gl) {
@@ -121,36 +122,59 @@ __global__ void __launch_bounds__(256, 4)
     });
     return;
   }
-  const int64_t b0 = (int64_t)(blockIdx.x - npiv_all) * kRowsPerBlock;
-  if (b0 + (threadIdx.x & ~31) / kGroup >= rows) return;  // whole warp past the end
-  const int64_t row = b0 + threadIdx.x / kGroup;
+  const int64_t row = (int64_t)(blockIdx.x - npiv_all) * RPB + threadIdx.x / TEAM;
+  if (row - (threadIdx.x & 31) / TEAM >= rows) return;  // whole warp past the end
   const bool valid = row < rows;
-  const int gl = lane & (kGroup - 1);
-  const int32_t start = valid ? __ldg(rp + row) : 0;
-  const int32_t len = valid ? __ldg(rl + row) : 0;
-  const int32_t blk = F == kFmtBlock4 && valid ? __ldg(ci.rblk + row) : 0;
-  float acc[RS];
+  const int t = threadIdx.x % T;                     // right-hand sides 4 t .. 4 t + 3
+  const int l0 = (threadIdx.x % TEAM) / T * V;       // first lane
+  const RowAt at = row_at<F>(row, valid, rp, rl, ci);
+  const float4* x4 = reinterpret_cast<const float4*>(xi) + t;
+  float acc[V][4];
 #pragma unroll
-  for (int r = 0; r < RS; ++r) acc[r] = 0.f;
-  for (int32_t e = gl * C; e < len; e += S) {
-    int32_t cs[C];
-    float v[C];
-    chunk_cols<F>(ci, start + e, e, blk, cs);
-    chunk_vals<VT, F>(val, start + e, v);
+  for (int v = 0; v < V; ++v)
 #pragma unroll
-    for (int i = 0; i < C; ++i) {
-      float xv[RS];
-      gather_rhs<RS>(xi, cs[i], xv);
+    for (int q = 0; q < 4; ++q) acc[v][q] = 0.f;
+  for (int32_t e = l0 * C; e < at.len; e += S) {
+    int32_t cs[V][C];
+    float a[V][C];
 #pragma unroll
-      for (int r = 0; r < RS; ++r) acc[r] = fmaf(v[i], xv[r], acc[r]);
+    for (int v = 0; v < V; ++v) {
+      if (v == 0 || e + v * C < at.len) {
+        chunk_cols<F>(ci, at.start + e + v * C, e, at.blk, cs[v]);
+        chunk_vals<VT, F>(val, at.start + e + v * C, a[v]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < C; ++i) {
+          cs[v][i] = 0;
+          a[v][i] = 0.f;
+        }
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+      if (v > 0 && e + v * C >= at.len) break;  // lane v has no chunk left
+#pragma unroll
+      for (int i = 0; i < C; ++i) {
+        const float4 xv = __ldg(x4 + (int64_t)cs[v][i] * T);
+        acc[v][0] = fmaf(a[v][i], xv.x, acc[v][0]);
+        acc[v][1] = fmaf(a[v][i], xv.y, acc[v][1]);
+        acc[v][2] = fmaf(a[v][i], xv.z, acc[v][2]);
+        acc[v][3] = fmaf(a[v][i], xv.w, acc[v][3]);
+      }
     }
   }
+  // the 16-lane butterfly: lanes 8, 4, 2, 1 apart
 #pragma unroll
-  for (int r = 0; r < RS; ++r) acc[r] = group_sum<kGroup>(acc[r]);
-  if (valid) {
+  for (int v = 0; v < V; ++v)
 #pragma unroll
-    for (int r = 0; r < RS; ++r)
-      if (r == gl && r < R) y[(int64_t)r * ystride + row] = acc[r];
+    for (int o = TEAM / 2; o >= T; o >>= 1)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) acc[v][q] += __shfl_xor_sync(0xffffffffu, acc[v][q], o);
+  if (!valid || l0 != 0) return;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float sum = V == 2 ? acc[0][q] + acc[V - 1][q] : acc[0][q];
+    if (4 * t + q < R) y[(int64_t)(4 * t + q) * ystride + row] = sum;
   }
 }
 
@@ -254,8 +278,8 @@ void launch_spmv_pivots(const DevCsr& A, int vt, const XT* x, YT* y, PivotCoef p
 template <typename VT, int RS>
 void spmm_typed(const DevCsr& A, const float* xi, float* y, int64_t ystride, int R,
                 const PivotCoef& pc, cudaStream_t s) {
-  const int64_t blocks =
-      (int64_t)pc.npiv_blocks * pc.nprob + (A.rows + kRowsPerBlock - 1) / kRowsPerBlock;
+  constexpr int kRows = RS == 4 ? 16 : 8;  // rows per block (k_spmm_pivots)
+  const int64_t blocks = (int64_t)pc.npiv_blocks * pc.nprob + (A.rows + kRows - 1) / kRows;
   const VT* v = reinterpret_cast<const VT*>(A.val);
   auto run = [&](auto F) {
     k_spmm_pivots<VT, RS, F.value><<<(unsigned)blocks, 256, 0, s>>>(
