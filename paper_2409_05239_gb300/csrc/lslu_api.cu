@@ -450,6 +450,17 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
   CT* u = (CT*)c->u;
   const int64_t ldh = c->kmax + 1, ldw = c->kmax;
   int64_t launches = 0;
+  // FP32 full searches leave their key to the scale pass (slot 0: L side, 1: D)
+  const bool keyed = std::is_same<CT, float>::value && nsamp == 0;
+  auto scale = [&](CT* v, BT* out, int64_t rows, const PivotArgs& pa, const int32_t* tp) {
+    if constexpr (std::is_same<CT, float>::value) {
+      if (keyed) {
+        launch_scale_pivot(v, out, rows, pa, c->st, s);
+        return;
+      }
+    }
+    launch_scale<CT, BT>(v, out, rows, c->st, P, tp, s, c->num_sms);
+  };
 
   if (k_begin == 0) {
   launch_init_state(c->st, P, K, s);
@@ -492,7 +503,7 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
   {
     PivotArgs pa{c->tp, c->kmax + 1, 0, c->tused, nullptr, 0, c->ldt, LSLU_BREAKDOWN_BETA,
                  0, 1, c->TDi, c->t_stride, c->coef, c->c_stride, P, tpm,
-                 fixed ? c->fixed_tp : nullptr, samp(0), nsamp, c->rank_m, c->unrank_m};
+                 fixed ? c->fixed_tp : nullptr, samp(0), nsamp, c->rank_m, c->unrank_m, -1};
     launch_init_pivot<BT>(c->r0, m, pa, c->st, s, c->num_sms);
     launch_scale<double, BT>(c->r0, D, m, c->st, P, tpm, s, c->num_sms);
     launches += 3;
@@ -523,10 +534,10 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
     PivotArgs paw{c->gp, c->kmax, k, c->gused, c->W + k + k * ldw, c->w_stride, c->ldt,
                   LSLU_BREAKDOWN_W, k, 0, c->TLi, c->t_stride, c->coef, c->c_stride, P, tpn,
                   fixed ? c->fixed_gp : nullptr, samp(2 * k + 1), nsamp, c->rank_n,
-                  c->unrank_n};
+                  c->unrank_n, keyed ? 0 : -1};
     launch_eliminate_argmax<CT, BT, CT>(q, L, c->ldl, k, n, q, paw, c->part_val, c->part_idx,
                                         c->part_cap, c->st, s, c->num_sms);
-    launch_scale<CT, BT>(q, L + (int64_t)k * c->ldl, n, c->st, P, tpn, s, c->num_sms);
+    scale(q, L + (int64_t)k * c->ldl, n, paw, tpn);
     // u = A l_k (with H(0:k+1, k)); eliminate d_0..d_k; pivot; d_{k+1}
     PivotCoef pch{c->tp,       c->kmax + 1,   k + 1,    D,          c->ldd,
                   c->coef,     c->c_stride,   c->H + k * ldh,       c->h_stride,
@@ -549,10 +560,10 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
     PivotArgs pah{c->tp, c->kmax + 1, k + 1, c->tused, c->H + (k + 1) + k * ldh, c->h_stride,
                   c->ldt, LSLU_BREAKDOWN_H, k, 0, c->TDi, c->t_stride, c->coef, c->c_stride, P,
                   tpm, fixed ? c->fixed_tp : nullptr, samp(2 * k + 2), nsamp, c->rank_m,
-                  c->unrank_m};
+                  c->unrank_m, keyed ? 1 : -1};
     launch_eliminate_argmax<CT, BT, CT>(u, D, c->ldd, k + 1, m, u, pah, c->part_val,
                                         c->part_idx, c->part_cap, c->st, s, c->num_sms);
-    launch_scale<CT, BT>(u, D + (int64_t)(k + 1) * c->ldd, m, c->st, P, tpm, s, c->num_sms);
+    scale(u, D + (int64_t)(k + 1) * c->ldd, m, pah, tpm);
     launches += 6;
   }
   }  // graph-mode basis loop

@@ -375,11 +375,15 @@ __global__ void __launch_bounds__(32)
       if (pa.nprob == 1) {
         bkey = tkey > bkey ? tkey : bkey;
       } else if (lane == 0 && tkey) {  // batch: one atomicMax per tile on its problem
-        atomicMax(&st[p].amax, tkey);
+        atomicMax(pa.key_slot >= 0 ? &st[p].key[pa.key_slot] : &st[p].amax, tkey);
       }
     }
   }
   if constexpr (kKey) {
+    if (pa.key_slot >= 0) {  // the scale pass takes the key from here
+      if (pa.nprob == 1 && lane == 0 && bkey) atomicMax(&st[0].key[pa.key_slot], bkey);
+      return;
+    }
     if (pa.nprob == 1 && lane == 0 && bkey) atomicMax(&st[0].amax, bkey);
     if (lane == 0) {
       __threadfence();
@@ -519,6 +523,58 @@ __global__ void k_scale(const CT* __restrict__ v, BT* __restrict__ out, int64_t 
     if (full || i0 + e < rows) out[i0 + e] = (BT)(a[e] / p);
 }
 
+// The same with the FP32 pivot still in the search's key: the key holds the
+// pivot's value, so every block scales at once, and one thread per problem
+// records the pivot meanwhile.  The elimination then ends with its atomicMax:
+// a fence, a ticket, the last block's exchange and record at its tail cost
+// every step 0.9 to 1.4 us of dependent L2 round trips (32x32 FP32 loop 12.2 ->
+// 10.8 us per half iteration, 256x256 0.9 us less, a 16-problem batch 4.6).
+__global__ void k_scale_pivot(const float* __restrict__ v, float* __restrict__ out, int64_t rows,
+                              PivotArgs pa, DevState* st) {
+  pdl_wait();  // v and the key come from the elimination before
+  pdl_trigger();
+  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t i0 = tid * 4;
+  if (i0 < rows) {
+    const bool full = i0 + 4 <= rows;
+    float a[4];
+    if (full) {
+      const float4 w = *reinterpret_cast<const float4*>(v + i0);
+      a[0] = w.x; a[1] = w.y; a[2] = w.z; a[3] = w.w;
+    } else {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) a[e] = i0 + e < rows ? v[i0 + e] : 0.f;
+    }
+    const int p = tile_problem(pa.tile_prob, i0);
+    const unsigned long long m = __ldcg(&st[p].key[pa.key_slot]);
+    const float pv = pa.fixed ? __ldcg(v + pa.fixed[(int64_t)p * pa.piv_stride + pa.piv_slot])
+                              : key_value(m);
+    // no pivot (breakdown, non-finite): what the recording thread finds too
+    if (__ldcg(&st[p].status) == LSLU_OK && pv != 0.f && isfinite(pv)) {
+#pragma unroll
+      for (int e = 0; e < 4; ++e) a[e] = a[e] / pv;
+      if (full) {
+        *reinterpret_cast<float4*>(out + i0) = make_float4(a[0], a[1], a[2], a[3]);
+      } else {
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (i0 + e < rows) out[i0 + e] = a[e];
+      }
+    }
+  }
+  if (tid < pa.nprob) {
+    const int p = (int)tid;
+    const unsigned long long m = __ldcg(&st[p].key[pa.key_slot]);
+    st[p].key[pa.key_slot ^ 1] = 0ull;  // for the next search; the last one's scale has read it
+    if (st[p].status == LSLU_OK) {
+      const int bi = m ? unrank_of(pa, key_index(m)) : -1;
+      const float a = __uint_as_float((unsigned)(m >> 32));
+      record_pivot<float, float>(pa, st[p], p, bi, (a != a) ? INFINITY : (double)a, v, true,
+                                 key_value(m));
+    }
+  }
+}
+
 __global__ void k_init_state(DevState* st, int nprob, int K) {
   for (int p = threadIdx.x; p < nprob; p += blockDim.x) {
     DevState& s = st[p];
@@ -531,6 +587,7 @@ __global__ void k_init_state(DevState* st, int nprob, int K) {
     s.pivot_f = 0.0f;
     s.amin = 0x7fffffff;
     s.amax = 0ull;
+    s.key[0] = s.key[1] = 0ull;
   }
 }
 
@@ -656,6 +713,12 @@ void launch_scale(const CT* v, BT* out, int64_t rows, DevState* st, int nprob,
   if (g < 1) return;
   launch_pdl(k_scale<CT, BT>, dim3((unsigned)g), dim3(kThreads), 0, s, v, out, rows, st, nprob,
              tile_prob);
+}
+
+void launch_scale_pivot(const float* v, float* out, int64_t rows, const PivotArgs& pa,
+                        DevState* st, cudaStream_t s) {
+  const int64_t g = (rows + 4 * kThreads - 1) / (4 * kThreads);
+  launch_pdl(k_scale_pivot, dim3((unsigned)g), dim3(kThreads), 0, s, v, out, rows, pa, st);
 }
 
 void launch_init_state(DevState* st, int nprob, int K, cudaStream_t s) {

@@ -122,6 +122,7 @@ struct DevState {
   float pivot_f;    // same, FP32 copy for the FP32 scale kernel
   int32_t amin;     // lowest index attaining the maximum (exact r0 pivot search)
   unsigned long long amax;  // running argmax key of the pivot search
+  unsigned long long key[2];  // FP32 pivot keys of the L-side / D-side searches
 };
 
 // Work space of the projected-problem kernel (global memory): one slot per
@@ -419,6 +420,9 @@ struct PivotArgs {
   // null: the row index itself)
   const int32_t* rank;
   const int32_t* unrank;
+  // FP32 searches over all rows: the pivot key goes to st[p].key[key_slot] and
+  // launch_scale_pivot resolves it; -1: the elimination's last block does
+  int key_slot;
 };
 
 template <typename XT, typename BT, typename CT>
@@ -435,6 +439,11 @@ void launch_init_pivot(const double* r0, int64_t rows, const PivotArgs& pa, DevS
 template <typename CT, typename BT>
 void launch_scale(const CT* v, BT* out, int64_t rows, DevState* st, int nprob,
                   const int32_t* tile_prob, cudaStream_t s, int num_sms);
+
+// out = v / pivot with the pivot taken from st[p].key[pa.key_slot] and recorded
+// (pivot list, mask, Hessenberg entry, state); clears the other slot.
+void launch_scale_pivot(const float* v, float* out, int64_t rows, const PivotArgs& pa,
+                        DevState* st, cudaStream_t s);
 
 void launch_residual0(const double* b, const double* Ax0, double* r0, int64_t m, cudaStream_t s);
 // G^(k) of Eq. (stop2) for k = 1..K from the projected residuals and traces
