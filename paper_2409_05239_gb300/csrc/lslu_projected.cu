@@ -126,29 +126,46 @@ __device__ void block_sum4(double (&v)[4], double* red4, int& parity) {
   for (int q = 0; q < 4; ++q) v[q] = __shfl_sync(0xffffffffu, t, 8 * q);
 }
 
+// q^-1/2 and 1 / d by one Halley iteration (third order: y (1 + e/2 + 3 e^2/8)
+// with e = 1 - q y^2; r (1 + e + e^2) with e = 1 - d r) on the hardware's
+// approximations of about 2^-20: within one unit of the last place of CUDA's
+// rsqrt and division on 2^-60 .. 2^60, without their calls and special cases
+// (arguments here are sums of squares and norms of scaled columns).
+__device__ __forceinline__ double inv_sqrt(double q) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(q));
+  const double e = fma(-(q * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double inverse(double d) {
+  double r;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(d));
+  const double e = fma(-d, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
 // Reflector I - tau v v^T (v0 = 1, v_rest = rest * scale) mapping
-// x = (x0, rest), ||rest||^2 = ss, to bh e1.
+// x = (x0, rest), ||rest||^2 = ss, to bh e1.  With q = x0^2 + ss and nrm =
+// sqrt(q): bh = -sign(x0) nrm, tau = (|x0| + nrm) / nrm and 1 / (x0 - bh) =
+// sign(x0) / (|x0| + nrm).  Every FP64 instruction holds the pipe for 64
+// cycles, so signs and the zero test are on the bits: about 1000 cycles
+// instead of 1300 with FP64 comparisons, rsqrt and a division.
 __device__ __forceinline__ void house(double x0, double ss, double& tau, double& bh,
                                       double& scale) {
-  if (ss == 0.0) {
-    tau = 0.0;
-    bh = x0;
-    scale = 0.0;
-    return;
-  }
-  // with q = x0^2 + ss and nrm = sqrt(q): bh = -sign(x0) nrm,
-  // tau = (bh - x0) / bh = (|x0| + nrm) / nrm and 1 / (x0 - bh) =
-  // sign(x0) / (|x0| + nrm); one rsqrt and one division (each costs about as
-  // much as seven dependent FP64 FMAs here, a sqrt ten)
+  const int sign = __double2hiint(x0) & (int)0x80000000;
+  const bool none = ((__double2hiint(ss) & 0x7fffffff) | __double2loint(ss)) == 0;
   const double q = fma(x0, x0, ss);
-  const double rn = rsqrt(q);
+  // sums of squares far outside the approximations' range take the functions
+  const int ex = (__double2hiint(q) >> 20) & 0x7ff;
+  const bool far = ex < 64 || ex > 1983;
+  const double rn = far ? rsqrt(q) : inv_sqrt(q);
   const double nrm = q * rn;
   const double d = fabs(x0) + nrm;
-  const bool neg = x0 < 0.0;
-  bh = neg ? nrm : -nrm;
-  tau = d * rn;
-  const double id = 1.0 / d;
-  scale = neg ? -id : id;
+  const double id = far ? 1.0 / d : inverse(d);
+  auto flip = [](double v, int s) { return __hiloint2double(__double2hiint(v) ^ s, __double2loint(v)); };
+  tau = none ? 0.0 : d * rn;
+  bh = none ? x0 : flip(nrm, sign ^ (int)0x80000000);
+  scale = none ? 0.0 : flip(id, sign);
 }
 
 // The lambda grid, sigma_1 10^(-14 + t / 16), t = 0 .. 256: a decade times a
@@ -654,6 +671,211 @@ __global__ void __launch_bounds__(kTB) k_bidiag(ProjArgs a, ProjWork w) {
     ts[1] = gtimer();
     for (int q = 0; q < 4; ++q) ts[8 + q] = tsec[q];
   }
+}
+
+// ---- 1'. the same with the matrix in registers ------------------------------
+// For k < 32 NR: warp v = rank + CL w of the 4 CL warps of a cluster owns the
+// columns c = v mod 4 CL (NC of them at most), lane l their rows l + 32 e.  A
+// step is bound by its chain of FP64 instructions (64 cycles each), so what
+// k_bidiag spends beyond it is cut: columns are updated, and their products
+// with the next row formed, without shared memory; a CTA adds its four warps'
+// partial products before they are published, so a cluster exchanges CL
+// vectors instead of 16 (2 threads per row add them for NR = 2); every warp
+// forms both reflectors itself from the summed products, without block-wide
+// reductions.  Two block barriers and one cluster barrier per step.  Partial
+// products are added in the order of the columns modulo 4 CL, so a size has
+// one result (launch_projected picks the form by the problem's size alone).
+// k = 50: 260 -> 182 us, 63: 332 -> 231; histories of k = 1..50: 330 -> 241.
+__device__ __forceinline__ void warp_sum4(double (&v)[4], int lane) {
+  const bool up = lane & 16, up8 = lane & 8;
+  double a0 = up ? v[2] : v[0], a1 = up ? v[3] : v[1];
+  a0 += __shfl_xor_sync(0xffffffffu, up ? v[0] : v[2], 16);
+  a1 += __shfl_xor_sync(0xffffffffu, up ? v[1] : v[3], 16);
+  double c = up8 ? a1 : a0;
+  c += __shfl_xor_sync(0xffffffffu, up8 ? a0 : a1, 8);
+  c += __shfl_xor_sync(0xffffffffu, c, 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  c += __shfl_xor_sync(0xffffffffu, c, 1);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = __shfl_sync(0xffffffffu, c, 8 * q);
+}
+
+template <int NR, int NC, int CL>
+__global__ void __launch_bounds__(kTB) k_bidiag_regs(ProjArgs a, ProjWork w) {
+  constexpr int R = 32 * NR;       // rows held
+  constexpr int NW = kTB / 32;     // warps per CTA
+  constexpr int TPR = kTB >= 2 * R ? 2 : 1;  // threads that add up one row
+  __shared__ double part[NW][R];   // the warps' partial products
+  __shared__ double xP[2][R];      // the CTA's, by step parity
+  __shared__ double xC[2][R];      // the owner's copy of the step's column
+  __shared__ double Ps[R], cjs[R];
+  __shared__ double rows[NW][NC + 1];  // one row's entry of every column, and of the reflector
+  cg::cluster_group cluster = cg::this_cluster();
+  const int rank = (int)cluster.block_rank();
+  const int local = blockIdx.x / CL, nlocal = gridDim.x / CL;
+  const int prob = w.prob0 + (w.desc ? nlocal - 1 - local : local);
+  const ProbInfo pi = prob_info(a, prob);
+  const int k = pi.k;
+  if (k == 0) return;  // every CTA of the cluster sees the same k: no barrier is left waiting
+  const Slots S = slot_of(w, pi);
+  const double* Hp = a.H + (int64_t)pi.p * a.strideH;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int v0 = rank + CL * warp;  // first column
+  double m[NC][NR];                 // columns v0 + 4 CL i, rows lane + 32 e
+#pragma unroll
+  for (int i = 0; i < NC; ++i) {
+    const int c = v0 + NW * CL * i;
+#pragma unroll
+    for (int e = 0; e < NR; ++e) {
+      const int r = lane + 32 * e;
+      m[i][e] = c < k && r <= k ? Hp[r + (int64_t)c * a.ldh] : 0.0;
+    }
+  }
+  // entry of row r (uniform) of a column, held by lane r mod 32 in register
+  // r / 32: that lane puts it into a word of its warp's for all to read.  (The
+  // predicated store is written out: from a branch per register the compiler
+  // makes an indexed array in local memory.)
+  auto put_row = [&](const double (&x)[NR], int r, double* word) {
+    const unsigned at = (unsigned)__cvta_generic_to_shared(word);
+#pragma unroll
+    for (int e = 0; e < NR; ++e)
+      asm volatile(
+          "{ .reg .pred p; setp.eq.s32 p, %0, %1; @p st.shared.f64 [%2], %3; }" ::"r"(r),
+          "r"(lane + 32 * e), "r"(at), "d"(x[e])
+          : "memory");
+  };
+  // What step jn needs from this CTA: products of the columns c > jn with
+  // their entries of row jn (row jn: the partial squared norm), and from the
+  // owner of column jn that column.
+  double xr[NC];  // the columns' entries of the step's row
+  auto publish = [&](int jn) {
+    double p[NR];
+#pragma unroll
+    for (int e = 0; e < NR; ++e) p[e] = 0.0;
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < NC; ++i) put_row(m[i], jn, &rows[warp][i]);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const int c = v0 + NW * CL * i;
+      xr[i] = rows[warp][i];
+      if (c > jn && c < k) {
+#pragma unroll
+        for (int e = 0; e < NR; ++e)
+          if (e >= jn >> 5) p[e] = fma(m[i][e], xr[i], p[e]);
+      }
+      if (c == jn)
+#pragma unroll
+        for (int e = 0; e < NR; ++e) xC[jn & 1][lane + 32 * e] = m[i][e];
+    }
+#pragma unroll
+    for (int e = 0; e < NR; ++e)
+      if (e >= jn >> 5) part[warp][lane + 32 * e] = p[e];
+    __syncthreads();
+    for (int r = (jn & ~31) + tid; r <= k; r += kTB)
+      xP[jn & 1][r] = (part[0][r] + part[2][r]) + (part[1][r] + part[3][r]);
+  };
+  publish(0);
+  for (int j = 0; j < k; ++j) {
+    const int par = j & 1, e0 = (j + 1) >> 5;
+    // Step j's vectors are complete in every CTA.  Those of parity par are
+    // rewritten only in step j+2, after the next barrier, which no CTA passes
+    // before all have read them below.
+    cluster.sync();
+    for (int r = (j & ~31) + tid / TPR; r <= (k | 31) && r < R; r += kTB / TPR) {
+      constexpr int Q = CL / TPR;
+      const int h = tid % TPR;  // TPR = 2: even and odd ranks
+      double pv[Q];
+#pragma unroll
+      for (int q = 0; q < Q; ++q)
+        pv[q] = *cluster.map_shared_rank(&xP[par][r], q * TPR + h);
+#pragma unroll
+      for (int o = Q / 2; o >= 1; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < o; ++q) pv[q] += pv[q + o];
+      if (TPR == 2) pv[0] += __shfl_xor_sync(0xffffffffu, pv[0], 1);
+      if (h == 0) Ps[r] = pv[0];
+      if (h == TPR - 1) cjs[r] = *cluster.map_shared_rank(&xC[par][r], j % CL);
+    }
+    __syncthreads();
+    // right reflector on row j, left reflector on column j, in every warp
+    double tr, bh, sc;
+    house(cjs[j], Ps[j], tr, bh, sc);
+    double s[NR], u[NR], s2 = 0.0;
+#pragma unroll
+    for (int e = 0; e < NR; ++e) {
+      s[e] = u[e] = 0.0;
+      if (e >= e0) {
+        const int r = lane + 32 * e;
+        const bool in = r > j && r <= k;
+        const double c = in ? cjs[r] : 0.0, p = in ? Ps[r] : 0.0;
+        s[e] = fma(sc, p, c);
+        u[e] = fma(-tr, s[e], c);
+        const double x = r >= j + 2 ? u[e] : 0.0;
+        s2 = fma(x, x, s2);
+      }
+    }
+    s2 = warp_sum_d(s2);
+    put_row(u, j + 1, &rows[warp][NC]);
+    __syncwarp();
+    double tl, bl, scl;
+    house(rows[warp][NC], s2, tl, bl, scl);
+#pragma unroll
+    for (int e = 0; e < NR; ++e)
+      if (e >= e0) u[e] = lane + 32 * e == j + 1 ? 1.0 : u[e] * scl;
+    if (rank == 0 && tid == 0) {
+      S.al[j] = bh;
+      S.be[j + 1] = bl;
+      S.taur[j] = tr;
+      S.Qs[(int64_t)j * k + j] = 1.0;
+    }
+    // own columns c > j: the right reflector, then the left one
+    constexpr int NT = (NC + 3) / 4 * 4;
+    double t[NT];
+#pragma unroll
+    for (int i = 0; i < NT; ++i) t[i] = 0.0;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const int c = v0 + NW * CL * i;
+      if (c > j && c < k) {
+        const double wc = xr[i] * sc;
+        if (lane == 0) __stcg(S.Qs + (int64_t)j * k + c, wc);
+        const double g = tr * wc;
+#pragma unroll
+        for (int e = 0; e < NR; ++e)
+          if (e >= e0) {
+            m[i][e] = fma(-g, s[e], m[i][e]);
+            t[i] = fma(u[e], m[i][e], t[i]);
+          }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NC; i += 4) {
+      if (v0 + NW * CL * (i + 3) > j) {  // not all of them are done
+        if (NC - i == 1) {
+          t[i] = warp_sum_d(t[i]);
+        } else {
+          double q[4] = {t[i], t[i + 1], t[i + 2], t[i + 3]};
+          warp_sum4(q, lane);
+          t[i] = q[0]; t[i + 1] = q[1]; t[i + 2] = q[2]; t[i + 3] = q[3];
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < NC; ++i) {
+      const int c = v0 + NW * CL * i;
+      if (c > j && c < k) {
+        const double h = tl * t[i];
+#pragma unroll
+        for (int e = 0; e < NR; ++e)
+          if (e >= e0) m[i][e] = fma(-h, u[e], m[i][e]);
+      }
+    }
+    if (j + 1 < k) publish(j + 1);
+  }
+  // no CTA leaves while another may still read its shared memory
+  cluster.sync();
 }
 
 // ---- 2. singular values and weights ----------------------------------------
@@ -1580,6 +1802,18 @@ int64_t projected_slot_doubles(int kk, int /*CL*/) {
   return 5 * (int64_t)(kk + 1) + kGrid + 1 + gram_doubles(kk) + (int64_t)kk * kk + (int64_t)(kk + 1) * kk + 64;
 }
 
+namespace {
+// Register-resident bidiagonalisations: the largest k of each and its cluster.
+// Beyond two registers per column the form loses its lead (measured against
+// k_bidiag: four rows and columns per lane 565 / 540 us at k = 100, eight rows
+// 1950 / 1532 at k = 200), so larger problems take k_bidiag.
+struct BidiagForm {
+  int kmax, cluster;
+  void (*kernel)(ProjArgs, ProjWork);
+};
+const BidiagForm kBidiagForms[] = {{63, 8, k_bidiag_regs<2, 2, 8>}};
+}  // namespace
+
 // Per-device set-up of the projected kernels: their attributes (cluster size
 // above 8, dynamic shared memory above 48 KB) are properties of the device
 // they are set on, so they are set once for every device the process uses,
@@ -1606,6 +1840,8 @@ ProjDeviceSetup setup_current_device() {
   if (cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     d.num_sms = 0;
   cudaFuncSetAttribute(k_bidiag, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  for (const BidiagForm& f : kBidiagForms)
+    cudaFuncSetAttribute(f.kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   cudaFuncSetAttribute(k_bidiag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap);
   cudaFuncSetAttribute(k_sigma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap);
   cudaFuncSetAttribute(k_sigma_lanes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap);
@@ -1638,6 +1874,49 @@ ProjDeviceSetup setup_current_device() {
 
 int projected_cluster_size() { return setup_current_device().cluster; }
 
+namespace {
+cudaError_t launch_clusters(void (*kernel)(ProjArgs, ProjWork), int CL, int count, size_t smem,
+                            const ProjArgs& a, const ProjWork& w, cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(count * CL), 1, 1);
+  cfg.blockDim = dim3(kTB, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = CL;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, a, w);
+}
+
+// k_bidiag for `count` problems of at most kcap columns.
+cudaError_t launch_bidiag_general(const ProjArgs& a, ProjWork& w, int kcap, int count, bool batch,
+                                  int num_sms, cudaStream_t s) {
+  const size_t K1 = (size_t)kcap + 1;
+  // shared memory: 5 + 2 kMaxCluster / cl vectors, and the slab of the CTA's
+  // columns when it fits beside them
+  auto vec_bytes = [&](int cl) { return (size_t)(5 + 2 * (kMaxCluster / cl)) * K1 * sizeof(double); };
+  auto slab_bytes = [&](int cl) { return (size_t)((kcap + cl - 1) / cl) * K1 * sizeof(double); };
+  // A history (problems of every size up to kcap) with more CTAs than two
+  // per SM keeps the GPU busy with many clusters at once: there 8 CTAs per
+  // problem do the whole batch in about 0.56 of the time 16 take (k = 1..300),
+  // although one problem alone is fastest on 16.
+  int CL = w.cluster;
+  if (!batch && count * CL > 2 * num_sms && CL > kHistoryCluster &&
+      vec_bytes(kHistoryCluster) + slab_bytes(kHistoryCluster) <= kSmemCap)
+    CL = kHistoryCluster;
+  const size_t vecs = vec_bytes(CL), slab = slab_bytes(CL);
+  w.kcap = kcap;
+  w.slab_in_smem = (vecs + slab <= kSmemCap) ? 1 : 0;
+  const size_t dyn = vecs + (w.slab_in_smem ? slab : 0);
+  if (dyn > kSmemCap) return cudaErrorInvalidValue;
+  return launch_clusters(k_bidiag, CL, count, dyn, a, w, s);
+}
+}  // namespace
+
 cudaError_t launch_projected(const ProjArgs& a, ProjWork& w, cudaStream_t s, int* nlaunch) {
   if (nlaunch) *nlaunch = 0;
   // one problem per k of k_first..k_last (histories), or one final problem
@@ -1651,44 +1930,35 @@ cudaError_t launch_projected(const ProjArgs& a, ProjWork& w, cudaStream_t s, int
   const ProjDeviceSetup dev_setup = setup_current_device();
   const int kmax = a.k_last;
   const size_t K1 = (size_t)kmax + 1;
-  // shared memory of k_bidiag: 5 + 2 kMaxCluster / cl vectors, and the slab
-  // of the CTA's columns when it fits beside them
-  auto vec_bytes = [&](int cl) { return (size_t)(5 + 2 * (kMaxCluster / cl)) * K1 * sizeof(double); };
-  auto slab_bytes = [&](int cl) { return (size_t)((kmax + cl - 1) / cl) * K1 * sizeof(double); };
-  // A history (problems of every size up to kmax) with more CTAs than two
-  // per SM keeps the GPU busy with many clusters at once: there 8 CTAs per
-  // problem, largest k first, do the whole batch in about 0.56 of the time 16
-  // take (k = 1..300), although one problem alone is fastest on 16.
-  int CL = w.cluster;
-  w.desc = 0;
-  if (!batch && nprob * CL > 2 * dev_setup.num_sms && CL > kHistoryCluster &&
-      vec_bytes(kHistoryCluster) + slab_bytes(kHistoryCluster) <= kSmemCap) {
-    CL = kHistoryCluster;
-    w.desc = 1;
-  }
-  w.prob0 = 0;
-  w.kcap = 0;
-  const size_t vecs = vec_bytes(CL), slab = slab_bytes(CL);
-  w.slab_in_smem = (vecs + slab <= kSmemCap) ? 1 : 0;
-  const size_t dyn1 = vecs + (w.slab_in_smem ? slab : 0);
   const size_t dyn2 = 4 * K1 * sizeof(double);
   const size_t dyn4 = 7 * K1 * sizeof(double);
-  if (dyn1 > kSmemCap || dyn2 > kSmemCap || dyn4 > kSmemCap) return cudaErrorInvalidValue;
-  // 1. bidiagonalisation, one cluster per problem
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(nprob * CL), 1, 1);
-  cfg.blockDim = dim3(kTB, 1, 1);
-  cfg.dynamicSmemBytes = dyn1;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CL;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, k_bidiag, a, w);
-  if (e != cudaSuccess) return e;
+  if (dyn2 > kSmemCap || dyn4 > kSmemCap) return cudaErrorInvalidValue;
+  // 1. bidiagonalisation, one cluster per problem, largest problems first.
+  // The form follows from a problem's size alone, so that a size has one
+  // result whether solved alone, in a batch or in a history.
+  int launches = 0;
+  const int small = batch ? kmax : a.k_first;  // sizes small .. kmax
+  for (int hi = kmax; hi >= small;) {
+    const BidiagForm* form = nullptr;  // null: k_bidiag
+    int lo = small;
+    for (const BidiagForm& f : kBidiagForms) {
+      if (hi <= f.kmax && f.cluster <= w.cluster) {
+        form = &f;
+        break;
+      }
+      if (f.cluster <= w.cluster) lo = lo > f.kmax + 1 ? lo : f.kmax + 1;
+    }
+    const int count = batch ? nprob : hi - lo + 1;
+    w.prob0 = batch ? 0 : lo - small;
+    w.desc = !batch && count > 1;
+    const cudaError_t e = form ? launch_clusters(form->kernel, form->cluster, count, 0, a, w, s)
+                               : launch_bidiag_general(a, w, hi, count, batch, dev_setup.num_sms, s);
+    if (e != cudaSuccess) return e;
+    ++launches;
+    hi = lo - 1;
+  }
+  w.prob0 = 0;
+  w.desc = 0;
   // 2. singular values and weights.  Final problems (the one of size k_last,
   // every batch entry) always take k_sigma, so that x does not depend on
   // whether histories were asked for or on the batch a problem was solved
@@ -1720,7 +1990,7 @@ cudaError_t launch_projected(const ProjArgs& a, ProjWork& w, cudaStream_t s, int
   }
   // 4. lambda, residual, y
   k_finish<<<(unsigned)nprob, kTF, dyn4, s>>>(a, w);
-  if (nlaunch) *nlaunch = 4 + (nlanes > 0 ? 1 : 0) + (grid ? 1 : 0);
+  if (nlaunch) *nlaunch = launches + 3 + (nlanes > 0 ? 1 : 0) + (grid ? 1 : 0);
   return cudaGetLastError();
 }
 
