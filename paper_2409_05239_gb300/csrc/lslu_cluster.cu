@@ -42,11 +42,11 @@ namespace {
 
 namespace cg = cooperative_groups;
 
-constexpr int kCT = 512;             // threads per CTA
-constexpr int kCW = kCT / 32;        // warps per CTA
+constexpr int kMaxCT = 640;          // threads per CTA: one pass over its rows where that fits
+constexpr int kMinCT = 256;
+constexpr int kAhead = 8;            // entries per lane in flight
 constexpr int kLanesPerRow = 4;      // lanes of one row of a product or an elimination
 constexpr int kSumLanes = 8;         // lanes of one coefficient or one new T^-1 entry
-constexpr int kRowsPerPass = kCT / kLanesPerRow;
 constexpr int kMaxClusterCTAs = 16;
 
 struct ClusterArgs {
@@ -119,15 +119,15 @@ __device__ __forceinline__ CT key_value(const PKey& k) {
 __device__ __forceinline__ int key_rank(const PKey& k) {
   return (int)(0x7fffffffu - (k.lo >> 1));
 }
-__device__ __forceinline__ PKey warp_max_key(PKey k, unsigned mask = 0xffffffffu) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    PKey x;
-    x.hi = __shfl_xor_sync(mask, k.hi, o);
-    x.lo = __shfl_xor_sync(mask, k.lo, o);
-    if (key_less(k, x)) k = x;
-  }
-  return k;
+// Word by word: the lanes that hold the largest upper words go on.
+__device__ __forceinline__ PKey warp_max_key(const PKey& k) {
+  const unsigned a = (unsigned)(k.hi >> 32), b = (unsigned)k.hi;
+  const unsigned ma = __reduce_max_sync(0xffffffffu, a);
+  const unsigned mb = __reduce_max_sync(0xffffffffu, a == ma ? b : 0u);
+  PKey r;
+  r.hi = ((unsigned long long)ma << 32) | mb;
+  r.lo = __reduce_max_sync(0xffffffffu, k.hi == r.hi ? k.lo : 0u);
+  return r;
 }
 
 template <typename VT>
@@ -158,7 +158,7 @@ __device__ __forceinline__ int owner_of(int64_t row, int64_t rows, int C) {
 // Shared-memory layout of one CTA (offsets in bytes).
 template <typename CT>
 struct CLayout {
-  size_t xv, rows_max, yown, vown, rp, rl, used, cs, xs, trow, slots_h, slots_l, gps, tps, tl, td,
+  size_t xv, rows_max, yown, vown, rp, rl, used, cs, xs, slots_h, slots_l, gps, tps, tl, td,
       lrows, drows, total;
   int ldr;  // leading dimension of the own basis rows (row-major, columns 0..K)
   int lds;
@@ -181,7 +181,7 @@ struct CLayout {
     used = take(2 * rows_max);
     cs = take(kc * sizeof(CT));
     xs = take(kc * sizeof(CT));
-    trow = take(kc * sizeof(CT));
+    take(kc * sizeof(CT));  // unused: the sizes served stay as documented
     slots_h = take(kMaxClusterCTAs * sizeof(unsigned long long));
     slots_l = take(kMaxClusterCTAs * sizeof(unsigned));
     gps = take(kc * sizeof(int32_t));
@@ -196,7 +196,7 @@ struct CLayout {
 };
 
 template <typename VT, typename BT, typename CT>
-__global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
+__global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   cg::cluster_group cluster = cg::this_cluster();
   const int C = (int)cluster.num_blocks();
@@ -210,7 +210,6 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
   uint8_t* used_s = smem + lay.used;
   CT* cs = reinterpret_cast<CT*>(smem + lay.cs);
   CT* xs = reinterpret_cast<CT*>(smem + lay.xs);
-  CT* trow = reinterpret_cast<CT*>(smem + lay.trow);
   unsigned long long* slot_h = reinterpret_cast<unsigned long long*>(smem + lay.slots_h);
   unsigned* slot_l = reinterpret_cast<unsigned*>(smem + lay.slots_l);
   CT* lrows = reinterpret_cast<CT*>(smem + lay.lrows);  // own rows of the bases, kept in
@@ -222,20 +221,20 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
   CT* TDs = reinterpret_cast<CT*>(smem + lay.td);
   const int lds = lay.lds;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  __shared__ int s_idx;
-  __shared__ CT s_piv;
+  const int nt = blockDim.x, nw = nt >> 5;
+  const int rows_per_pass = nt / kLanesPerRow;
 
   // own rows: m-space [m0, m1), n-space [n0, n1)
   const int64_t m0 = range_lo(a.m, me, C), m1 = range_lo(a.m, me + 1, C);
   const int64_t n0 = range_lo(a.n, me, C), n1 = range_lo(a.n, me + 1, C);
   const int nm = (int)(m1 - m0), nn = (int)(n1 - n0);
   const size_t rmax = lay.rows_max;
-  for (int i = tid; i < nm; i += kCT) {
+  for (int i = tid; i < nm; i += nt) {
     rp_s[i] = __ldg(a.a_rp + m0 + i);
     rl_s[i] = __ldg(a.a_rl + m0 + i);
     used_s[i] = 0;
   }
-  for (int i = tid; i < nn; i += kCT) {
+  for (int i = tid; i < nn; i += nt) {
     rp_s[rmax + i] = __ldg(a.t_rp + n0 + i);
     rl_s[rmax + i] = __ldg(a.t_rl + n0 + i);
     used_s[rmax + i] = 0;
@@ -248,8 +247,8 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
 
   // the CTA's largest key over the keys every thread holds, written into
   // slot `me` of every CTA of the cluster
-  __shared__ unsigned long long w_hi[kCW];
-  __shared__ unsigned w_lo[kCW];
+  __shared__ unsigned long long w_hi[kMaxCT / 32];
+  __shared__ unsigned w_lo[kMaxCT / 32];
   auto publish_key = [&](PKey k) {
     k = warp_max_key(k);
     if (lane == 0) {
@@ -259,8 +258,8 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
     __syncthreads();
     if (warp == 0) {
       PKey b;
-      b.hi = lane < kCW ? w_hi[lane] : 0ull;
-      b.lo = lane < kCW ? w_lo[lane] : 0u;
+      b.hi = lane < nw ? w_hi[lane] : 0ull;
+      b.lo = lane < nw ? w_lo[lane] : 0u;
       b = warp_max_key(b);
       if (lane < C) {  // lane q sends the CTA's best to CTA q
         *cluster.map_shared_rank(slot_h + me, lane) = b.hi;
@@ -269,25 +268,18 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
     }
   };
   // the cluster-wide pivot from the C slots (after a cluster barrier), the
-  // same in every CTA: rank into s_idx (-1: none), value into s_piv
-  auto resolve_slots = [&]() {
-    if (warp == 0) {
-      PKey b;
-      b.hi = lane < C ? slot_h[lane] : 0ull;
-      b.lo = lane < C ? slot_l[lane] : 0u;
-      b = warp_max_key(b);
-      if (lane == 0) {
-        s_idx = (b.hi | b.lo) ? key_rank(b) : -1;
-        s_piv = key_value<CT>(b);
-      }
-    }
-    __syncthreads();
+  // same in every thread of every CTA
+  auto resolve_slots = [&]() -> PKey {
+    PKey b;
+    b.hi = lane < C ? slot_h[lane] : 0ull;
+    b.lo = lane < C ? slot_l[lane] : 0u;
+    return warp_max_key(b);
   };
 
   // ---- pivot of r0 (exact, FP64) and d_1 = r0 / beta
   {
     PKey best = {0ull, 0u};
-    for (int i = tid; i < nm; i += kCT) {
+    for (int i = tid; i < nm; i += nt) {
       if (__ldg(a.tused + m0 + i)) {  // (single problem: nothing is pivoted yet)
         used_s[i] = 1;
         continue;
@@ -298,21 +290,9 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
     }
     publish_key(best);
     cluster.sync();
-    // the exact FP64 pivot of r0 (resolve_slots gives the compute type)
-    __shared__ double s_beta;
-    if (warp == 0) {
-      PKey b;
-      b.hi = lane < C ? slot_h[lane] : 0ull;
-      b.lo = lane < C ? slot_l[lane] : 0u;
-      b = warp_max_key(b);
-      if (lane == 0) {
-        s_idx = (b.hi | b.lo) ? key_rank(b) : -1;
-        s_beta = key_value<double>(b);
-      }
-    }
-    __syncthreads();
-    const int rk = s_idx;
-    const double beta = s_beta;
+    const PKey b = resolve_slots();
+    const int rk = (b.hi | b.lo) ? key_rank(b) : -1;
+    const double beta = key_value<double>(b);
     const int idx = rk >= 0 ? (a.unrank_m ? __ldg(a.unrank_m + rk) : rk) : -1;
     if (idx < 0 || beta == 0.0 || !isfinite(beta)) {
       if (me == 0 && tid == 0) {
@@ -337,7 +317,7 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
     }
     // d_1 on the own rows: the global basis, the own rows of D and every
     // CTA's input copy
-    for (int i = tid; i < nm; i += kCT) {
+    for (int i = tid; i < nm; i += nt) {
       const BT d = (BT)(__ldg(a.r0 + m0 + i) / beta);
       Db[m0 + i] = d;
       drows[(size_t)i * ldr] = (CT)d;
@@ -346,6 +326,26 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
     cluster.sync();
   }
 
+  // The first kAhead entries per lane of a thread's row of the next product:
+  // the matrix does not change, so they are requested half an iteration ahead
+  // and the product starts with its gathers.
+  int32_t ac[kAhead];
+  CT av[kAhead];
+  auto load_entries = [&](const int32_t* col, const VT* val, int32_t st, int32_t len, int32_t e) {
+#pragma unroll
+    for (int u = 0; u < kAhead; ++u) {
+      const int32_t q = e + u * kLanesPerRow;
+      ac[u] = q < len ? __ldg(col + st + q) : -1;
+      av[u] = q < len ? (CT)val_at<VT>(val, st + q) : (CT)0;
+    }
+  };
+  auto load_first = [&](bool Ls) {  // of the first pass over the rows of a side
+    const int rr = tid / kLanesPerRow;
+    const bool in = rr < (Ls ? nn : nm);
+    const int32_t st = in ? rp_s[Ls ? rmax + rr : rr] : 0, len = in ? rl_s[Ls ? rmax + rr : rr] : 0;
+    load_entries(Ls ? a.t_col : a.a_col, Ls ? tval : aval, st, len, tid & (kLanesPerRow - 1));
+  };
+  load_first(true);
   for (int k = 0; k < a.K; ++k) {
     for (int side = 0; side < 2; ++side) {
       // side 0: q = A^T d_k against L (n-space rows); side 1: u = A l_k
@@ -364,27 +364,17 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
       CT* brows = Ls ? lrows : drows;  // own rows of this side's basis
       CT* Ts = Ls ? TLs : TDs;
       // ---- P1: own rows of the product, gathering from the input copy
-      for (int base = 0; base < nr; base += kRowsPerPass) {
+      for (int base = 0; base < nr; base += rows_per_pass) {
         const int rr = base + tid / kLanesPerRow;
         const int gl = tid & (kLanesPerRow - 1);
         CT acc = 0, acc2 = 0;
-        if (rr < nr) {
-          const int32_t st = rps[rr], len = rls[rr];
-          // eight entries per lane in flight: loads first, then the gathers
-          for (int32_t e = gl; e < len; e += 8 * kLanesPerRow) {
-            int32_t cc[8];
-            CT vv[8];
+        const int32_t st = rr < nr ? rps[rr] : 0, len = rr < nr ? rls[rr] : 0;
+        for (int32_t e = gl; e < len; e += kAhead * kLanesPerRow) {
+          if (base > 0 || e != gl) load_entries(col, val, st, len, e);
 #pragma unroll
-            for (int u = 0; u < 8; ++u) {
-              const int32_t q = e + u * kLanesPerRow;
-              cc[u] = q < len ? __ldg(col + st + q) : -1;
-              vv[u] = q < len ? (CT)val_at<VT>(val, st + q) : (CT)0;
-            }
-#pragma unroll
-            for (int u = 0; u < 8; u += 2) {
-              if (cc[u] >= 0) acc = fma(vv[u], xv[cc[u]], acc);
-              if (cc[u + 1] >= 0) acc2 = fma(vv[u + 1], xv[cc[u + 1]], acc2);
-            }
+          for (int u = 0; u < kAhead; u += 2) {
+            if (ac[u] >= 0) acc = fma(av[u], xv[ac[u]], acc);
+            if (ac[u + 1] >= 0) acc2 = fma(av[u + 1], xv[ac[u + 1]], acc2);
           }
         }
         acc += acc2;
@@ -392,9 +382,10 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
         for (int o = kLanesPerRow / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (rr < nr && gl == 0) yown[rr] = acc;
       }
+      load_first(!Ls);
       cluster.sync();
       // ---- P2: coefficients c = T^-1 y(piv), y at the pivot rows from their owners
-      for (int j = tid; j < cnt; j += kCT) {
+      for (int j = tid; j < cnt; j += nt) {
         const int64_t pr = piv[j];
         const int o = owner_of(pr, rows, C);
         xs[j] = *cluster.map_shared_rank(yown + (pr - range_lo(rows, o, C)), o);
@@ -403,7 +394,7 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
       // (kSumLanes lanes per coefficient, each a strided part of its sum, then
       // a fixed shuffle tree: the dependent FP64 chains are kSumLanes times
       // shorter and spread over the CTA's warps)
-      for (int b0 = 0; b0 < cnt; b0 += kCT / kSumLanes) {
+      for (int b0 = 0; b0 < cnt; b0 += nt / kSumLanes) {
         const int i = b0 + tid / kSumLanes, part = tid & (kSumLanes - 1);
         CT sum = 0;
         if (i < cnt)
@@ -415,12 +406,12 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
       __syncthreads();
       if (me == 0) {
         double* hess = Ls ? a.W + (int64_t)k * a.ldw : a.H + (int64_t)k * a.ldh;
-        for (int j = tid; j < cnt; j += kCT) hess[j] = (double)cs[j];
+        for (int j = tid; j < cnt; j += nt) hess[j] = (double)cs[j];
       }
       // ---- P3: eliminate the own rows (lane group per row, columns split
       // over the group's lanes in a fixed order), then the CTA's best
       PKey best = {0ull, 0u};
-      for (int base = 0; base < nr; base += kRowsPerPass) {
+      for (int base = 0; base < nr; base += rows_per_pass) {
         const int rr = base + tid / kLanesPerRow;
         const int gl = tid & (kLanesPerRow - 1);
         CT acc = 0, acc2 = 0;
@@ -451,11 +442,11 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
       publish_key(best);
       cluster.sync();
       // ---- P4: the pivot, T^-1, the new basis vector
-      resolve_slots();
-      const int rk = s_idx;
+      const PKey best_key = resolve_slots();
+      const int rk = (best_key.hi | best_key.lo) ? key_rank(best_key) : -1;
       const int32_t* unrank = Ls ? a.unrank_n : a.unrank_m;
       const int idx = rk >= 0 ? (unrank ? __ldg(unrank + rk) : rk) : -1;
-      const CT pv = s_piv;
+      const CT pv = key_value<CT>(best_key);
       const int slot = cnt;
       if (idx < 0 || pv == (CT)0 || !isfinite((double)pv)) {
         if (me == 0 && tid == 0) {
@@ -483,40 +474,35 @@ __global__ void __launch_bounds__(kCT, 1) k_cluster_basis(ClusterArgs a) {
           (Ls ? a.gused : a.tused)[idx] = 1;
         }
       }
-      // new row `slot` of T^-1: T(slot, l) = b_l(idx), from the owner's rows
-      {
-        const int o = owner_of(idx, rows, C);
-        const CT* orow =
-            cluster.map_shared_rank(brows, o) + (size_t)(idx - range_lo(rows, o, C)) * ldr;
-        for (int l = tid; l < slot; l += kCT) trow[l] = orow[l];
-      }
-      __syncthreads();
-      // (kSumLanes lanes per entry j, each a strided part of the sum over
-      // l = j .. slot-1, then a fixed shuffle tree; the terms l < j are zero)
-      for (int b0 = 0; b0 < slot; b0 += kCT / kSumLanes) {
-        const int j = b0 + tid / kSumLanes, part = tid & (kSumLanes - 1);
-        CT sum = 0;
-        if (j < slot)
-          for (int l = j + part; l < slot; l += kSumLanes) sum = fma(trow[l], Ts[j * lds + l], sum);
-#pragma unroll
-        for (int o = kSumLanes / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-        if (j < slot && part == 0) Ts[j * lds + slot] = -sum;
-      }
-      if (tid == 0) Ts[slot * lds + slot] = (CT)1;
-      __syncthreads();
-      if (me == 0) {
-        CT* Tg = reinterpret_cast<CT*>(Ls ? a.TLi : a.TDi);
-        for (int j = tid; j <= slot; j += kCT) Tg[(int64_t)j * a.ldt + slot] = Ts[j * lds + slot];
-      }
       // b_new = v / pivot on the own rows: the global basis (column k of L, or
       // k+1 of D) and every CTA's input copy for the next product
       BT* out = Ls ? Lb + (int64_t)k * a.ldl : Db + (int64_t)(k + 1) * a.ldd;
       const int ocol = Ls ? k : k + 1;
-      for (int i = tid; i < nr; i += kCT) {
+      for (int i = tid; i < nr; i += nt) {
         const BT b = (BT)(vown[i] / pv);
         out[r0 + i] = b;
         brows[(size_t)i * ldr + ocol] = (CT)b;
         for (int q = 0; q < C; ++q) *cluster.map_shared_rank(xv + r0 + i, q) = (CT)b;
+      }
+      // new row `slot` of T^-1, T(slot, l) = b_l(idx) from the owner's rows: CTA
+      // c forms the entries j = c mod C, a warp each, and writes them into every
+      // CTA's copy (read two half iterations on).  Every CTA forming the whole
+      // row took 3400 cycles of a half iteration's 24000.
+      {
+        const int o = owner_of(idx, rows, C);
+        const CT* orow =
+            cluster.map_shared_rank(brows, o) + (size_t)(idx - range_lo(rows, o, C)) * ldr;
+        CT* Tg = reinterpret_cast<CT*>(Ls ? a.TLi : a.TDi);
+        for (int j = me + C * warp; j < slot; j += C * nw) {
+          CT sum = 0;
+          for (int l = j + lane; l < slot; l += 32) sum = fma(orow[l], Ts[j * lds + l], sum);
+#pragma unroll
+          for (int of = 16; of > 0; of >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, of);
+          if (lane < C) *cluster.map_shared_rank(Ts + j * lds + slot, lane) = -sum;
+          if (lane == 0) Tg[(int64_t)j * a.ldt + slot] = -sum;
+        }
+        if (tid == 0) Ts[slot * lds + slot] = (CT)1;
+        if (me == 0 && tid == 0) Tg[(int64_t)slot * a.ldt + slot] = (CT)1;
       }
       cluster.sync();
     }
@@ -543,7 +529,7 @@ int setup_typed() {
   for (int cand : {16, 8}) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cand);
-    cfg.blockDim = dim3(kCT);
+    cfg.blockDim = dim3(kMaxCT);
     cfg.dynamicSmemBytes = kClusterSmemCap;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -625,7 +611,10 @@ cudaError_t launch_cluster_basis(Ctx* c, const double* r0, int K, int C, cudaStr
   a.K = K;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)C);
-  cfg.blockDim = dim3(kCT);
+  // a thread group per row in one pass where that fits
+  const int64_t rows_max = (std::max(a.m, a.n) + C - 1) / C;
+  const int64_t want = (rows_max * kLanesPerRow + 31) / 32 * 32;
+  cfg.blockDim = dim3((unsigned)std::min<int64_t>(kMaxCT, std::max<int64_t>(kMinCT, want)));
   cfg.stream = s;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
