@@ -13,13 +13,13 @@
 // (release / acquire):
 //
 //   P1  y = A^T d_k (or A l_k) on the CTA's own rows, gathering from its copy
-//       of the input vector;                                   cluster barrier
-//   P2  coefficients c = T^-1 y(piv): y at the pivot rows read from the owning
-//       CTAs; P3  eliminate the own rows, v = y - B c (0 on pivoted rows), and
-//       send the CTA's largest |v| (value, rank) to every CTA;  cluster barrier
-//   P4  every CTA reduces the C candidates in CTA order (the same pivot
-//       everywhere), extends its T^-1, stores b_new = v / pivot on its own rows
-//       and writes them into every CTA's copy of the input vector;
+//       of the input vector; y at the pivot rows goes to every CTA;
+//                                                               cluster barrier
+//   P2  coefficients c = T^-1 y(piv); P3  eliminate the own rows, v = y - B c
+//       (0 on pivoted rows), and send the CTA's largest |v| (value, rank) to every CTA;  cluster barrier
+//   P4  every warp reduces the C candidates (the same pivot everywhere), the CTA
+//       stores b_new = v / pivot on its own rows, writes them into every CTA's
+//       copy of the input vector, and forms its share of the new row of T^-1;
 //                                                               cluster barrier
 //
 // The matrix stays in global memory (L2-resident at these sizes); the bases
@@ -48,6 +48,9 @@ constexpr int kAhead = 8;            // entries per lane in flight
 constexpr int kLanesPerRow = 4;      // lanes of one row of a product or an elimination
 constexpr int kSumLanes = 8;         // lanes of one coefficient or one new T^-1 entry
 constexpr int kMaxClusterCTAs = 16;
+// used_s of a row: 0, its pivot slot + 1 (K stays below 200: two (K+1)^2
+// matrices fit in shared memory), or kMasked (never a pivot)
+constexpr int kMasked = 255;
 
 struct ClusterArgs {
   int64_t m, n;
@@ -146,19 +149,20 @@ __device__ __forceinline__ double val_at<__nv_bfloat16>(const __nv_bfloat16* p, 
 }
 
 // Row range [lo, hi) of CTA c among C over `rows` rows.
-__device__ __forceinline__ int64_t range_lo(int64_t rows, int c, int C) {
-  return rows * c / C;
+// (32-bit arithmetic: the rows fit in shared memory)
+__device__ __forceinline__ int range_lo(int rows, int c, int C) {
+  return (int)((unsigned)rows * (unsigned)c / (unsigned)C);
 }
-__device__ __forceinline__ int owner_of(int64_t row, int64_t rows, int C) {
+__device__ __forceinline__ int owner_of(int row, int rows, int C) {
   // largest c with rows * c / C <= row
-  int c = (int)(((row + 1) * C - 1) / rows);
+  const int c = (int)((((unsigned)row + 1) * (unsigned)C - 1) / (unsigned)rows);
   return c < C ? c : C - 1;
 }
 
 // Shared-memory layout of one CTA (offsets in bytes).
 template <typename CT>
 struct CLayout {
-  size_t xv, rows_max, yown, vown, rp, rl, used, cs, xs, slots_h, slots_l, gps, tps, tl, td,
+  size_t xv, rows_max, yown, vown, rp, rl, used, cs, xs, slots_h, slots_l, tl, td,
       lrows, drows, total;
   int ldr;  // leading dimension of the own basis rows (row-major, columns 0..K)
   int lds;
@@ -181,11 +185,10 @@ struct CLayout {
     used = take(2 * rows_max);
     cs = take(kc * sizeof(CT));
     xs = take(kc * sizeof(CT));
-    take(kc * sizeof(CT));  // unused: the sizes served stay as documented
     slots_h = take(kMaxClusterCTAs * sizeof(unsigned long long));
     slots_l = take(kMaxClusterCTAs * sizeof(unsigned));
-    gps = take(kc * sizeof(int32_t));
-    tps = take(kc * sizeof(int32_t));
+    o += (kc * sizeof(CT) + 15) / 16 * 16 + 2 * ((kc * sizeof(int32_t) + 15) / 16 * 16);
+    // (unused: the sizes that fit stay what they were)
     tl = take((size_t)(K + 1) * lds * sizeof(CT));
     td = take((size_t)(K + 1) * lds * sizeof(CT));
     ldr = K + 1 + (((K + 1) & 1) ? 0 : 1);
@@ -215,8 +218,6 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
   CT* lrows = reinterpret_cast<CT*>(smem + lay.lrows);  // own rows of the bases, kept in
   CT* drows = reinterpret_cast<CT*>(smem + lay.drows);  // shared memory (row-major)
   const int ldr = lay.ldr;
-  int32_t* gps = reinterpret_cast<int32_t*>(smem + lay.gps);  // pivot lists, the same in
-  int32_t* tps = reinterpret_cast<int32_t*>(smem + lay.tps);  // every CTA
   CT* TLs = reinterpret_cast<CT*>(smem + lay.tl);
   CT* TDs = reinterpret_cast<CT*>(smem + lay.td);
   const int lds = lay.lds;
@@ -225,9 +226,10 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
   const int rows_per_pass = nt / kLanesPerRow;
 
   // own rows: m-space [m0, m1), n-space [n0, n1)
-  const int64_t m0 = range_lo(a.m, me, C), m1 = range_lo(a.m, me + 1, C);
-  const int64_t n0 = range_lo(a.n, me, C), n1 = range_lo(a.n, me + 1, C);
-  const int nm = (int)(m1 - m0), nn = (int)(n1 - n0);
+  const int ma = (int)a.m, na = (int)a.n;
+  const int m0 = range_lo(ma, me, C), m1 = range_lo(ma, me + 1, C);
+  const int n0 = range_lo(na, me, C), n1 = range_lo(na, me + 1, C);
+  const int nm = m1 - m0, nn = n1 - n0;
   const size_t rmax = lay.rows_max;
   for (int i = tid; i < nm; i += nt) {
     rp_s[i] = __ldg(a.a_rp + m0 + i);
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
     PKey best = {0ull, 0u};
     for (int i = tid; i < nm; i += nt) {
       if (__ldg(a.tused + m0 + i)) {  // (single problem: nothing is pivoted yet)
-        used_s[i] = 1;
+        used_s[i] = kMasked;
         continue;
       }
       const int r = a.rank_m ? __ldg(a.rank_m + m0 + i) : (int)(m0 + i);
@@ -309,9 +311,8 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
     }
     if (tid == 0) {
       TDs[0] = (CT)1;
-      tps[0] = idx;
       if (idx >= m0 && idx < m1) {
-        used_s[idx - m0] = 1;
+        used_s[idx - m0] = 1;  // slot 0
         a.tused[idx] = 1;
       }
     }
@@ -352,21 +353,20 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
       // against D (m-space rows)
       const bool Ls = side == 0;
       const int nr = Ls ? nn : nm;
-      const int64_t r0 = Ls ? n0 : m0;
-      const int64_t rows = Ls ? a.n : a.m;
+      const int r0 = Ls ? n0 : m0;
+      const int rows = Ls ? na : ma;
+      const int rr0 = tid / kLanesPerRow, gl = tid & (kLanesPerRow - 1);
       const int32_t* rps = Ls ? rp_s + rmax : rp_s;
       const int32_t* rls = Ls ? rl_s + rmax : rl_s;
       uint8_t* us = Ls ? used_s + rmax : used_s;
       const int32_t* col = Ls ? a.t_col : a.a_col;
       const VT* val = Ls ? tval : aval;
       const int cnt = Ls ? k : k + 1;  // earlier basis vectors of this side
-      const int32_t* piv = Ls ? gps : tps;
       CT* brows = Ls ? lrows : drows;  // own rows of this side's basis
       CT* Ts = Ls ? TLs : TDs;
       // ---- P1: own rows of the product, gathering from the input copy
       for (int base = 0; base < nr; base += rows_per_pass) {
-        const int rr = base + tid / kLanesPerRow;
-        const int gl = tid & (kLanesPerRow - 1);
+        const int rr = base + rr0;
         CT acc = 0, acc2 = 0;
         const int32_t st = rr < nr ? rps[rr] : 0, len = rr < nr ? rls[rr] : 0;
         for (int32_t e = gl; e < len; e += kAhead * kLanesPerRow) {
@@ -381,16 +381,13 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
 #pragma unroll
         for (int o = kLanesPerRow / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         if (rr < nr && gl == 0) yown[rr] = acc;
+        const int sl = rr < nr ? us[rr] : 0;  // a pivot row: its y goes to every CTA
+        if (sl > 0 && sl < kMasked)
+          for (int q = gl; q < C; q += kLanesPerRow) *cluster.map_shared_rank(xs + sl - 1, q) = acc;
       }
       load_first(!Ls);
       cluster.sync();
-      // ---- P2: coefficients c = T^-1 y(piv), y at the pivot rows from their owners
-      for (int j = tid; j < cnt; j += nt) {
-        const int64_t pr = piv[j];
-        const int o = owner_of(pr, rows, C);
-        xs[j] = *cluster.map_shared_rank(yown + (pr - range_lo(rows, o, C)), o);
-      }
-      __syncthreads();
+      // ---- P2: coefficients c = T^-1 y(piv)
       // (kSumLanes lanes per coefficient, each a strided part of its sum, then
       // a fixed shuffle tree: the dependent FP64 chains are kSumLanes times
       // shorter and spread over the CTA's warps)
@@ -412,8 +409,7 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
       // over the group's lanes in a fixed order), then the CTA's best
       PKey best = {0ull, 0u};
       for (int base = 0; base < nr; base += rows_per_pass) {
-        const int rr = base + tid / kLanesPerRow;
-        const int gl = tid & (kLanesPerRow - 1);
+        const int rr = base + rr0;
         CT acc = 0, acc2 = 0;
         if (rr < nr) {
           const CT* bp = brows + (size_t)rr * ldr;
@@ -431,9 +427,9 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
           const CT v = us[rr] ? (CT)0 : yown[rr] - acc;
           vown[rr] = v;
           if (!us[rr]) {
-            const int64_t row = r0 + rr;
-            const int rk = Ls ? (a.rank_n ? __ldg(a.rank_n + row) : (int)row)
-                              : (a.rank_m ? __ldg(a.rank_m + row) : (int)row);
+            const int row = r0 + rr;
+            const int rk = Ls ? (a.rank_n ? __ldg(a.rank_n + row) : row)
+                              : (a.rank_m ? __ldg(a.rank_m + row) : row);
             const PKey kk = make_key<CT>(v, rk);
             if (key_less(best, kk)) best = kk;
           }
@@ -468,9 +464,8 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
         a.st[0].pivot_f = (float)pv;
       }
       if (tid == 0) {
-        (Ls ? gps : tps)[slot] = idx;
         if (idx >= r0 && idx < r0 + nr) {
-          us[idx - r0] = 1;
+          us[idx - r0] = (uint8_t)(slot + 1);
           (Ls ? a.gused : a.tused)[idx] = 1;
         }
       }
