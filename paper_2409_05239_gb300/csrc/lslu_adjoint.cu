@@ -305,10 +305,14 @@ __global__ void __launch_bounds__(kT) k_adj_dots(DotArgs a) {
   extern __shared__ unsigned char smem_raw2[];
   double* r = reinterpret_cast<double*>(smem_raw2);  // reuses the v area (cnt doubles)
   __syncthreads();
-  for (int j = threadIdx.x; j < a.cnt; j += blockDim.x) {
+  // a warp per sum, lanes over the blocks' partials: one thread adding the ~300
+  // partials of a sum was a chain of FP64 additions of 64 cycles, 9 of the
+  // kernel's 17 us
+  for (int j = warp; j < a.cnt; j += kNW) {
     double s = 0.0;
-    for (int b = 0; b < (int)gridDim.x; ++b) s += __ldcg(a.part + (int64_t)b * a.ldp + j);
-    r[j] = (a.ext ? a.ext[j] : 0.0) + a.sgn * s;
+    for (int b = lane; b < (int)gridDim.x; b += 32) s += __ldcg(a.part + (int64_t)b * a.ldp + j);
+    s = warp_sum(s);
+    if (lane == 0) r[j] = (a.ext ? a.ext[j] : 0.0) + a.sgn * s;
   }
   __syncthreads();
   if (!a.Tinv) {
@@ -317,13 +321,20 @@ __global__ void __launch_bounds__(kT) k_adj_dots(DotArgs a) {
   }
   const BT* Ti = reinterpret_cast<const BT*>(a.Tinv);
   CT* sc = reinterpret_cast<CT*>(a.store_c);
-  for (int i = threadIdx.x; i < a.cnt; i += blockDim.x) {
+  for (int i0 = 0; i0 < a.cnt; i0 += kT / 8) {  // eight lanes per entry
+    const int i = i0 + threadIdx.x / 8, part = threadIdx.x & 7;
     double s = 0.0;
-    const BT* col = Ti + (int64_t)i * a.ldt;
-    for (int l = i; l < a.cnt; ++l) s += (double)col[l] * r[l];
-    a.out_vec[i] = s;
-    const int32_t row = a.piv[i];
-    __stcg(sc + row, (CT)((double)__ldcg(sc + row) + s));
+    if (i < a.cnt) {
+      const BT* col = Ti + (int64_t)i * a.ldt;
+      for (int l = i + part; l < a.cnt; l += 8) s += (double)col[l] * r[l];
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (i < a.cnt && part == 0) {
+      a.out_vec[i] = s;
+      const int32_t row = a.piv[i];
+      __stcg(sc + row, (CT)((double)__ldcg(sc + row) + s));
+    }
   }
 }
 
@@ -332,13 +343,20 @@ __global__ void __launch_bounds__(kT) k_adj_dots(DotArgs a) {
 //   Hbar = (beta e1 - H y) ztil^T - (H ztil) y^T, betabar = (H ztil)_0,
 //   lambdabar = -2 lambda ztil^T y.
 constexpr int kPT = 1024;
+constexpr size_t kAdjSmemCap = 200 * 1024;
 
 __global__ void __launch_bounds__(kPT)
     k_adj_projected(const double* __restrict__ H, int64_t ldh, int K, const double* y,
-                    const DevState* st, const double* lam_ptr, const double* ybar, double* M,
-                    double* zt, double* Hbar, double* scal) {
+                    const DevState* st, const double* lam_ptr, const double* ybar, double* Mg,
+                    double* zt_out, double* Hbar, double* scal, int in_smem) {
+  // M and ztil in shared memory where they fit: every column of the factor
+  // waits for the one before, and in global memory each of those steps took
+  // several L2 round trips
+  extern __shared__ double msh[];
   __shared__ double red[kPT / 32];
   __shared__ int bad;
+  double* M = in_smem ? msh : Mg;
+  double* zt = in_smem ? msh + (int64_t)K * K : zt_out;
   const double lam = *lam_ptr;
   const double beta = st->beta;
   const int tid = threadIdx.x;
@@ -405,8 +423,11 @@ __global__ void __launch_bounds__(kPT)
     __syncthreads();
   }
   // rH = beta e1 - H y and Hz = H ztil (length K+1), kept in M's space
-  double* rH = M;
-  double* Hz = M + (K + 1);
+  if (in_smem) {
+    for (int i = tid; i < K; i += blockDim.x) zt_out[i] = zt[i];
+  }
+  double* rH = Mg;
+  double* Hz = Mg + (K + 1);
   for (int r = tid; r <= K; r += blockDim.x) {
     double a1 = (r == 0) ? beta : 0.0, a2 = 0.0;
     for (int j = max(r - 1, 0); j < K; ++j) {
@@ -596,8 +617,14 @@ lslu_status adjoint_impl(Ctx* c, const double* xbar, double* bbar, double* lam_b
     a.st = c->st;
     launch_dots<BT, CT>(c, a, s);
   }
-  k_adj_projected<<<1, kPT, 0, s>>>(c->H, ldh, K, c->y, c->st, lam_ptr, ybar, sm + SL.M,
-                                    sm + SL.zt, Hbar, scal);
+  const size_t proj_smem = ((size_t)K * K + K) * sizeof(double);
+  const bool in_smem = proj_smem <= kAdjSmemCap &&
+                       cudaFuncSetAttribute(k_adj_projected,
+                                            cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)kAdjSmemCap) == cudaSuccess;
+  k_adj_projected<<<1, kPT, in_smem ? proj_smem : 0, s>>>(c->H, ldh, K, c->y, c->st, lam_ptr, ybar,
+                                                          sm + SL.M, sm + SL.zt, Hbar, scal,
+                                                          in_smem ? 1 : 0);
   launches += 3;
 
   for (int k = K - 1; k >= 0; --k) {
