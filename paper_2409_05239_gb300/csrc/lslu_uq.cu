@@ -36,7 +36,10 @@ namespace {
 
 constexpr int kTG = 64;    // Gram output tile (kTG x kTG)
 constexpr int kRC = 32;    // rows staged per step
-constexpr int kSlicesMax = 64;
+// Row slices of one Gram tile: FP32 products are summed in FP32 within a slice
+// (64 slices at most); FP64 ones take as many as fill the GPU's FP64 pipes.
+template <typename BT>
+constexpr int kSlicesMax = sizeof(BT) == 8 ? 152 : 64;
 
 // Partial Gram tiles: block (pair, slice) adds B1(r, i) B2(r, j) over its rows
 // for the kTG x kTG tile (ti, tj) of the pair list; 256 threads, 4 x 4 outputs
@@ -45,7 +48,7 @@ template <typename BT>
 __global__ void __launch_bounds__(256)
     k_gram_tiles(const BT* __restrict__ B1, int cols1, const BT* __restrict__ B2, int cols2,
                  int64_t ld, int64_t rows, const int2* __restrict__ pairs, int rows_per_slice,
-                 double* __restrict__ part) {
+                 int symmetric, double* __restrict__ part) {
   using CT = BT;  // accumulate in the basis type within a slice
   __shared__ BT s1[kRC][kTG + 1];
   __shared__ BT s2[kRC][kTG + 1];
@@ -54,6 +57,12 @@ __global__ void __launch_bounds__(256)
   const int64_t r_begin = (int64_t)blockIdx.y * rows_per_slice;
   const int64_t r_end = r_begin + rows_per_slice < rows ? r_begin + rows_per_slice : rows;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // 16 x 16 threads
+  // 16 x 16 sub-blocks past the columns, and below a symmetric tile's diagonal,
+  // are left out: an FP64 instruction holds the pipe for 64 cycles (k = 40:
+  // 496 -> 238 us per launch)
+  const int n1 = min(4, (cols1 - i0 + 15) / 16), n2 = min(4, (cols2 - j0 + 15) / 16);
+  const bool diag = symmetric && i0 == j0;
+  const bool whole = n1 == 4 && n2 == 4 && !diag;
   CT acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
@@ -84,18 +93,34 @@ __global__ void __launch_bounds__(256)
     }
     __syncthreads();
     if (r0 + kRC < r_end) fetch(r0 + kRC);
+    if (whole) {
 #pragma unroll 4
-    for (int rr = 0; rr < kRC; ++rr) {
-      CT a[4], b[4];
+      for (int rr = 0; rr < kRC; ++rr) {
+        CT a[4], b[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        a[q] = s1[rr][ty + 16 * q];
-        b[q] = s2[rr][tx + 16 * q];
+        for (int q = 0; q < 4; ++q) {
+          a[q] = s1[rr][ty + 16 * q];
+          b[q] = s2[rr][tx + 16 * q];
+        }
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[p][q] = fma(a[p], b[q], acc[p][q]);
       }
+    } else {
+      for (int rr = 0; rr < kRC; ++rr) {
+        CT a[4], b[4];
 #pragma unroll
-      for (int p = 0; p < 4; ++p)
+        for (int q = 0; q < 4; ++q) {
+          a[q] = s1[rr][ty + 16 * q];
+          b[q] = s2[rr][tx + 16 * q];
+        }
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = fma(a[p], b[q], acc[p][q]);
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (p < n1 && q < n2 && (!diag || q >= p)) acc[p][q] = fma(a[p], b[q], acc[p][q]);
+      }
     }
     __syncthreads();
   }
@@ -118,6 +143,8 @@ __global__ void k_gram_reduce(const double* __restrict__ part, const int2* __res
     const int w = (int)(e % (kTG * kTG));
     const int i = pairs[pi].x * kTG + w / kTG, j = pairs[pi].y * kTG + w % kTG;
     if (i >= cols1 || j >= cols2) continue;
+    // a symmetric tile's sub-blocks below its diagonal come from above it
+    if (symmetric && pairs[pi].x == pairs[pi].y && j / 16 < i / 16) continue;
     double s = 0.0;
     for (int sl = 0; sl < nslices; ++sl) s += part[((int64_t)sl * npairs + pi) * (kTG * kTG) + w];
     C[(int64_t)j * ldc + i] = s;
@@ -306,6 +333,7 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[p][q] = 0;
   const int bmax = k < a0 + kTG ? k : a0 + kTG;  // Ri(a, b) = 0 for b > a
+  const int nq = min(4, (k - a0 + 15) / 16);       // 16-entry groups inside the k entries
   for (int b0 = 0; b0 < bmax; b0 += kRC) {
     for (int e = threadIdx.x; e < kRC * kTG; e += blockDim.x) {
       // consecutive threads on consecutive rows of L (and entries a of Ri):
@@ -318,8 +346,9 @@ __global__ void __launch_bounds__(256)
       sr[bb][cc] = (b < k && a < k) ? Ri[(int64_t)b * k + a] : (BT)0;
     }
     __syncthreads();
+    const int nb = bmax - b0 < kRC ? bmax - b0 : kRC;  // (the rest is zero)
 #pragma unroll 4
-    for (int bb = 0; bb < kRC; ++bb) {
+    for (int bb = 0; bb < nb; ++bb) {
       CT x[4], y[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
@@ -329,7 +358,8 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) acc[p][q] = fma(x[p], y[q], acc[p][q]);
+        for (int q = 0; q < 4; ++q)
+          if (q < nq) acc[p][q] = fma(x[p], y[q], acc[p][q]);
     }
     __syncthreads();
   }
@@ -385,7 +415,7 @@ cudaError_t gram(const BT* B1, int cols1, const BT* B2, int cols2, int64_t ld, i
   for (int i = 0; i < t1; ++i)
     for (int j = symmetric ? i : 0; j < t2; ++j) pairs.push_back(make_int2(i, j));
   const int np = (int)pairs.size();
-  int nsl = std::max(1, std::min(kSlicesMax, (960 + np - 1) / np));
+  int nsl = std::max(1, std::min(kSlicesMax<BT>, (960 + np - 1) / np));
   while (nsl > 1 && (int64_t)nsl * np * kTG * kTG > part_cap) --nsl;
   if ((int64_t)nsl * np * kTG * kTG > part_cap) return cudaErrorInvalidValue;
   int64_t rps = (rows + nsl - 1) / nsl;
@@ -393,7 +423,7 @@ cudaError_t gram(const BT* B1, int cols1, const BT* B2, int cols2, int64_t ld, i
   cudaError_t e = cudaMemcpyAsync(dpairs, pairs.data(), np * sizeof(int2), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   k_gram_tiles<BT><<<dim3(np, nsl), 256, 0, s>>>(B1, cols1, B2, cols2, ld, rows, dpairs, (int)rps,
-                                                part);
+                                                symmetric ? 1 : 0, part);
   const int64_t tot = (int64_t)np * kTG * kTG;
   k_gram_reduce<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 4096), 256, 0, s>>>(
       part, dpairs, np, nsl, cols1, cols2, symmetric ? 1 : 0, C, ldc);
