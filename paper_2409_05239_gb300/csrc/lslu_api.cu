@@ -423,6 +423,8 @@ void collect_spmv_times(Ctx* c, int pairs) {
   cudaGetLastError();
 }
 
+constexpr int kDeferCoefs = 64;
+
 // Enqueues one whole solve on stream s (no host synchronisation, capturable):
 // state reset, r0 and its pivot, K basis iterations, the projected problems
 // and x = x0 + L y.  Inputs are read from the handle's staging buffers.
@@ -450,6 +452,17 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
   CT* u = (CT*)c->u;
   const int64_t ldh = c->kmax + 1, ldw = c->kmax;
   int64_t launches = 0;
+  // coefficient sums left to the elimination: one small problem with few
+  // earlier vectors, where every block of it adds a handful of partials instead
+  // of waiting for the product's last pivot block (a fence, a ticket and another
+  // read).  32x32 FP32 with histories, K = 50: 1881 -> 1743 us; a product that
+  // streams its matrix hides that wait (FP64 160x160 would take 1.5% longer,
+  // 256x256 0.5%).
+  auto part = [&](int cnt) -> const void* {
+    return P == 1 && cnt > 0 && cnt <= kDeferCoefs && c->A.nnz_padded < kStreamMinEntries
+               ? c->xp
+               : nullptr;
+  };
   // FP32 full searches leave their key to the scale pass (slot 0: L side, 1: D)
   const bool keyed = std::is_same<CT, float>::value && nsamp == 0;
   auto scale = [&](CT* v, BT* out, int64_t rows, const PivotArgs& pa, const int32_t* tp) {
@@ -503,7 +516,7 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
   {
     PivotArgs pa{c->tp, c->kmax + 1, 0, c->tused, nullptr, 0, c->ldt, LSLU_BREAKDOWN_BETA,
                  0, 1, c->TDi, c->t_stride, c->coef, c->c_stride, P, tpm,
-                 fixed ? c->fixed_tp : nullptr, samp(0), nsamp, c->rank_m, c->unrank_m, -1};
+                 fixed ? c->fixed_tp : nullptr, samp(0), nsamp, c->rank_m, c->unrank_m, -1, nullptr, 0, nullptr};
     launch_init_pivot<BT>(c->r0, m, pa, c->st, s, c->num_sms);
     launch_scale<double, BT>(c->r0, D, m, c->st, P, tpm, s, c->num_sms);
     launches += 3;
@@ -516,7 +529,7 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
     PivotCoef pcw{c->gp,       c->kmax,       k,        L,          c->ldl,
                   c->coef,     c->c_stride,   c->W + k * ldw,       c->w_stride,
                   c->xp,       c->xp_stride,  c->TLi,   c->ldt,     c->t_stride,
-                  c->st,       P,             0};
+                  c->st,       P,             0,        part(k) != nullptr};
     record_spmv_start(c, s, capturing, &e0);
     if constexpr (std::is_same<BT, float>::value) {
       if (c->shared_rhs) {
@@ -534,7 +547,7 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
     PivotArgs paw{c->gp, c->kmax, k, c->gused, c->W + k + k * ldw, c->w_stride, c->ldt,
                   LSLU_BREAKDOWN_W, k, 0, c->TLi, c->t_stride, c->coef, c->c_stride, P, tpn,
                   fixed ? c->fixed_gp : nullptr, samp(2 * k + 1), nsamp, c->rank_n,
-                  c->unrank_n, keyed ? 0 : -1};
+                  c->unrank_n, keyed ? 0 : -1, part(k), c->ldt, c->W + k * ldw};
     launch_eliminate_argmax<CT, BT, CT>(q, L, c->ldl, k, n, q, paw, c->part_val, c->part_idx,
                                         c->part_cap, c->st, s, c->num_sms);
     scale(q, L + (int64_t)k * c->ldl, n, paw, tpn);
@@ -542,7 +555,7 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
     PivotCoef pch{c->tp,       c->kmax + 1,   k + 1,    D,          c->ldd,
                   c->coef,     c->c_stride,   c->H + k * ldh,       c->h_stride,
                   c->xp,       c->xp_stride,  c->TDi,   c->ldt,     c->t_stride,
-                  c->st,       P,             0};
+                  c->st,       P,             0,        part(k + 1) != nullptr};
     record_spmv_start(c, s, capturing, &e0);
     if constexpr (std::is_same<BT, float>::value) {
       if (c->shared_rhs) {
@@ -560,7 +573,7 @@ int64_t enqueue_solve(Ctx* c, cudaStream_t s, const double* db, const double* dx
     PivotArgs pah{c->tp, c->kmax + 1, k + 1, c->tused, c->H + (k + 1) + k * ldh, c->h_stride,
                   c->ldt, LSLU_BREAKDOWN_H, k, 0, c->TDi, c->t_stride, c->coef, c->c_stride, P,
                   tpm, fixed ? c->fixed_tp : nullptr, samp(2 * k + 2), nsamp, c->rank_m,
-                  c->unrank_m, keyed ? 1 : -1};
+                  c->unrank_m, keyed ? 1 : -1, part(k + 1), c->ldt, c->H + k * ldh};
     launch_eliminate_argmax<CT, BT, CT>(u, D, c->ldd, k + 1, m, u, pah, c->part_val,
                                         c->part_idx, c->part_cap, c->st, s, c->num_sms);
     scale(u, D + (int64_t)(k + 1) * c->ldd, m, pah, tpm);

@@ -272,7 +272,17 @@ __global__ void __launch_bounds__(32)
     }
     if (p != cur_p) {  // the problem's coefficients (x and the flags are in flight meanwhile)
       __syncwarp();
-      for (int j = lane; j < cnt; j += 32) c[j] = (CT)pa.coef[(int64_t)p * pa.coef_stride + j];
+      if (pa.part) {
+        const CT* part = reinterpret_cast<const CT*>(pa.part);
+        for (int j = lane; j < cnt; j += 32) {
+          CT s = 0;
+          for (int b = 0; b <= j / 8; ++b) s += __ldcg(part + (int64_t)b * pa.part_ld + j);
+          c[j] = s;
+          if (t == 0 && status0 == LSLU_OK) pa.hess_col[j] = (double)s;
+        }
+      } else {
+        for (int j = lane; j < cnt; j += 32) c[j] = (CT)pa.coef[(int64_t)p * pa.coef_stride + j];
+      }
       __syncwarp();
       cur_p = p;
     }

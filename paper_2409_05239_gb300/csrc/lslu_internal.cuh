@@ -89,6 +89,14 @@ inline bool shape_cmp(int sh) {
   return (sh >= kShapesPerFormat && sh < kShapeE8) || (sh >= kShapeE8 && (sh & 1));
 }
 
+// Entries (with padding) from which the default FP32 / BF16 products read
+// 16-bit offsets with four chunks in flight (stream_rows).  Below, the matrix
+// stays in L2 and a product is a few dependent round trips, where the extra
+// base read and the wider step cost more than the bytes: a pair of products
+// 8.2 us either way up to 0.4 M entries, 12.4 against 14.6 us at 1.35 M, 18.4
+// against 22.0 at 3.2 M; a 32x32 solve (0.05 M) 2.20 against 2.15 ms.
+constexpr int64_t kStreamMinEntries = 1 << 20;
+
 struct DevCsr {
   int shape = kShapeG16U2;
   int compressed = 0;          // 16-bit column offsets available (off, ubase)
@@ -316,6 +324,7 @@ struct PivotCoef {
   DevState* st;
   int nprob;
   int npiv_blocks;   // per problem, set by the launcher
+  int defer;         // 1: leave the partial sums to the elimination (PivotArgs::part)
 };
 template <typename XT, typename YT>
 void launch_spmv_pivots(const DevCsr& A, int vt, const XT* x, YT* y, PivotCoef pc,
@@ -423,6 +432,12 @@ struct PivotArgs {
   // FP32 searches over all rows: the pivot key goes to st[p].key[key_slot] and
   // launch_scale_pivot resolves it; -1: the elimination's last block does
   int key_slot;
+  // single problems with few earlier vectors: the coefficients' partial sums of
+  // the product's pivot blocks (8 columns each, leading dimension part_ld),
+  // added by the elimination, whose first block writes hess_col; null: coef
+  const void* part;
+  int64_t part_ld;
+  double* hess_col;
 };
 
 template <typename XT, typename BT, typename CT>

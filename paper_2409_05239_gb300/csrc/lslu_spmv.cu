@@ -216,14 +216,6 @@ bool native(int vt) {
 
 }  // namespace
 
-// Entries (with padding) from which the default FP32 / BF16 products read
-// 16-bit offsets with four chunks in flight (stream_rows).  Below, the matrix
-// stays in L2 and a product is a few dependent round trips, where the extra
-// base read and the wider step cost more than the bytes: a pair of products
-// 8.2 us either way up to 0.4 M entries, 12.4 against 14.6 us at 1.35 M, 18.4
-// against 22.0 at 3.2 M; a 32x32 solve (0.05 M) 2.20 against 2.15 ms.
-constexpr int64_t kStreamMinEntries = 1 << 20;
-
 // Native products (FP64 vectors for FP64 values, FP32 otherwise) run in the
 // matrix's shape and column format; the others (FP64 vectors on FP32 / BF16
 // values: r0 with x0, the adjoint's x0 term) in the default shape.

@@ -448,7 +448,8 @@ __global__ void __launch_bounds__(256, (resident_blocks<VT, G, U, F>()))
 //   b. computes y(piv_j) with the same row reduction as every other row
 //      (so the two agree bit for bit);
 //   c. the block adds Tinv(i, j) y(piv_j) over its 8 columns into a partial
-//      vector; the last pivot block to finish adds the partials in block order.
+//      vector; the last pivot block to finish adds the partials in block order
+//      (pc.defer: the elimination does, in the same order).
 // The remaining blocks compute the other rows of y meanwhile.  rowdot(p, row,
 // gl) is the product of output row `row` for problem p.
 template <typename YT, int G, typename RowDot>
@@ -493,6 +494,7 @@ __device__ __forceinline__ void pivot_blocks(const PivotCoef& pc, RowDot rowdot)
       if (i >= j0 + w) acc = fma(__ldcg(Tinv + (int64_t)(j0 + w) * pc.ldi + i), xs[w], acc);
     __stcg(part + (int64_t)bb * pc.ldi + i, acc);
   }
+  if (pc.defer) return;
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) last = (atomicAdd(&sp.ticket2, 1) == pc.npiv_blocks - 1);
