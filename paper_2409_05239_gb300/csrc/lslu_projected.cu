@@ -1573,7 +1573,10 @@ __global__ void __launch_bounds__(kTF) k_finish(ProjArgs a, ProjWork w) {
         // the geometric midpoint), the bracket narrowed by the slope's sign;
         // it ends when a step moves mu by less than 1e-13 relative (near the
         // root the slope is rounding noise, and steps below that only wander
-        // inside it) or cannot move it at all
+        // inside it) or cannot move it at all.  A Newton step that leaves mu
+        // where it is has converged too: mu is then an end of the bracket, and
+        // the midpoint taken in its place would start over far from the root
+        // (one such problem kept a history's launch at 126 us instead of 25)
         double a2 = lo * lo, b2 = hi * hi, mu = lo * hi;
         for (int it = 0; it < 60; ++it) {
           const SlopeAndDerivative sd = gcv_slope2(sig2, c2, k, mu, omega, red4, par);
@@ -1583,6 +1586,7 @@ __global__ void __launch_bounds__(kTF) k_finish(ProjArgs a, ProjWork w) {
           else
             b2 = mu;
           double nx = (sd.ds > 0.0) ? mu - sd.s / sd.ds : -1.0;
+          if (nx == mu && isfinite(sd.ds)) break;
           if (!(nx > a2 && nx < b2)) nx = sqrt(a2) * sqrt(b2);
           if (!(nx > a2 && nx < b2) || nx == mu) break;
           const bool done = fabs(nx - mu) <= 1e-13 * mu;
