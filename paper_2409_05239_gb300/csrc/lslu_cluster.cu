@@ -480,21 +480,33 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
         for (int q = 0; q < C; ++q) *cluster.map_shared_rank(xv + r0 + i, q) = (CT)b;
       }
       // new row `slot` of T^-1, T(slot, l) = b_l(idx) from the owner's rows: CTA
-      // c forms the entries j = c mod C, a warp each, and writes them into every
-      // CTA's copy (read two half iterations on).  Every CTA forming the whole
-      // row took 3400 cycles of a half iteration's 24000.
+      // c forms the entries j = c mod C, kSumLanes lanes each, and writes them
+      // into every CTA's copy (read two half iterations on).  Every CTA forming
+      // the whole row took 3400 cycles of a half iteration's 24000.  An entry's
+      // lanes and their tree are fixed: a sum over a whole warp (two terms a lane
+      // instead of seven at K = 50) rounds otherwise, and the recurrence carries
+      // a last bit here to 1e-7 of H within 26 iterations (816 x 484, FP64).
       {
         const int o = owner_of(idx, rows, C);
         const CT* orow =
             cluster.map_shared_rank(brows, o) + (size_t)(idx - range_lo(rows, o, C)) * ldr;
         CT* Tg = reinterpret_cast<CT*>(Ls ? a.TLi : a.TDi);
-        for (int j = me + C * warp; j < slot; j += C * nw) {
+        constexpr int kEntries = 32 / kSumLanes;  // of a warp
+        // (from the last warp down: the first ones are at their rows' divisions)
+        for (int q0 = kEntries * (nw - 1 - warp); me + C * q0 < slot; q0 += kEntries * nw) {
+          const int j = me + C * (q0 + lane / kSumLanes), part = lane & (kSumLanes - 1);
           CT sum = 0;
-          for (int l = j + lane; l < slot; l += 32) sum = fma(orow[l], Ts[j * lds + l], sum);
+          if (j < slot)
+            for (int l = j + part; l < slot; l += kSumLanes)
+              sum = fma(orow[l], Ts[j * lds + l], sum);
 #pragma unroll
-          for (int of = 16; of > 0; of >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, of);
-          if (lane < C) *cluster.map_shared_rank(Ts + j * lds + slot, lane) = -sum;
-          if (lane == 0) Tg[(int64_t)j * a.ldt + slot] = -sum;
+          for (int of = kSumLanes / 2; of > 0; of >>= 1)
+            sum += __shfl_xor_sync(0xffffffffu, sum, of);
+          if (j < slot) {
+            for (int q = part; q < C; q += kSumLanes)
+              *cluster.map_shared_rank(Ts + j * lds + slot, q) = -sum;
+            if (part == 0) Tg[(int64_t)j * a.ldt + slot] = -sum;
+          }
         }
         if (tid == 0) Ts[slot * lds + slot] = (CT)1;
         if (me == 0 && tid == 0) Tg[(int64_t)slot * a.ldt + slot] = (CT)1;
