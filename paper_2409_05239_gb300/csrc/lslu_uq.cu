@@ -36,6 +36,13 @@ namespace {
 
 constexpr int kTG = 64;    // Gram output tile (kTG x kTG)
 constexpr int kRC = 32;    // rows staged per step
+// An FP64 instruction holds its pipe for 64 cycles, so the FP64 passes skip what
+// lies outside the columns; the FP32 ones are bound by their shared-memory reads
+// and lose more to the guards than they save (row pass and Gram tiles, 262144
+// rows, k = 300: 8.2 ms per call with them, 6.7 without).
+template <typename BT>
+constexpr bool kSkipOutside = sizeof(BT) == 8;
+
 // Row slices of one Gram tile: FP32 products are summed in FP32 within a slice
 // (64 slices at most); FP64 ones take as many as fill the GPU's FP64 pipes.
 template <typename BT>
@@ -62,7 +69,7 @@ __global__ void __launch_bounds__(256)
   // 496 -> 238 us per launch)
   const int n1 = min(4, (cols1 - i0 + 15) / 16), n2 = min(4, (cols2 - j0 + 15) / 16);
   const bool diag = symmetric && i0 == j0;
-  const bool whole = n1 == 4 && n2 == 4 && !diag;
+  const bool whole = !kSkipOutside<BT> || (n1 == 4 && n2 == 4 && !diag);
   CT acc[4][4];
 #pragma unroll
   for (int a = 0; a < 4; ++a)
@@ -346,7 +353,8 @@ __global__ void __launch_bounds__(256)
       sr[bb][cc] = (b < k && a < k) ? Ri[(int64_t)b * k + a] : (BT)0;
     }
     __syncthreads();
-    const int nb = bmax - b0 < kRC ? bmax - b0 : kRC;  // (the rest is zero)
+    // (the rest is zero)
+    const int nb = kSkipOutside<BT> && bmax - b0 < kRC ? bmax - b0 : kRC;
 #pragma unroll 4
     for (int bb = 0; bb < nb; ++bb) {
       CT x[4], y[4];
@@ -359,7 +367,7 @@ __global__ void __launch_bounds__(256)
       for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q)
-          if (q < nq) acc[p][q] = fma(x[p], y[q], acc[p][q]);
+          if (!kSkipOutside<BT> || q < nq) acc[p][q] = fma(x[p], y[q], acc[p][q]);
     }
     __syncthreads();
   }
