@@ -245,7 +245,9 @@ __global__ void __launch_bounds__(kMaxCT, 1) k_cluster_basis(ClusterArgs a) {
   BT* Db = reinterpret_cast<BT*>(a.D);
   const VT* aval = reinterpret_cast<const VT*>(a.a_val);
   const VT* tval = reinterpret_cast<const VT*>(a.t_val);
-  __syncthreads();
+  // every CTA has started before the first store into its shared memory (the
+  // r0 pivot's keys below; each later store follows a cluster barrier)
+  cluster.sync();
 
   // the CTA's largest key over the keys every thread holds, written into
   // slot `me` of every CTA of the cluster
