@@ -542,8 +542,9 @@ lslu_status ensure_workspace(Ctx* c) {
                 std::string("adjoint work space: ") + cudaGetErrorString(e));
   }
   c->adj_part_rows = (int)nblk_max;
-  cudaMemset(c->adj_Vb, 0, (size_t)c->ldl * K * bb);
-  cudaMemset(c->adj_Zb, 0, (size_t)c->ldd * K * bb);
+  if ((e = cudaMemsetAsync(c->adj_Vb, 0, (size_t)c->ldl * K * bb, c->stream)) != cudaSuccess ||
+      (e = cudaMemsetAsync(c->adj_Zb, 0, (size_t)c->ldd * K * bb, c->stream)) != cudaSuccess)
+    return fail(c, LSLU_ERR_CUDA, std::string("adjoint work space: ") + cudaGetErrorString(e));
   return LSLU_OK;
 }
 

@@ -145,15 +145,17 @@ lslu_status create_common(lslu_ctx* c, const int64_t* rp, const int32_t* ci, con
   c->xp_stride = (int64_t)((K + 8) / 8 + 1) * (K + 1);
   CKC(cudaMalloc(&c->L, (size_t)c->ldl * K * bb));
   CKC(cudaMalloc(&c->D, (size_t)c->ldd * (K + 1) * bb));
-  CKC(cudaMemset(c->L, 0, (size_t)c->ldl * K * bb));
-  CKC(cudaMemset(c->D, 0, (size_t)c->ldd * (K + 1) * bb));
+  // (zeroing on the handle's own stream: one that does not wait for the legacy
+  // stream would not see memsets there finished)
+  CKC(cudaMemsetAsync(c->L, 0, (size_t)c->ldl * K * bb, c->stream));
+  CKC(cudaMemsetAsync(c->D, 0, (size_t)c->ldd * (K + 1) * bb, c->stream));
   CKC(dmalloc(&c->H, (size_t)P * c->h_stride));
   CKC(dmalloc(&c->W, (size_t)P * c->w_stride));
   // a solve writes the upper Hessenberg part of H (triangle of W) only, and
   // the projected solve and lslu_get_state read whole columns: what cudaMalloc
   // left below must be zero
-  CKC(cudaMemset(c->H, 0, (size_t)P * c->h_stride * sizeof(double)));
-  CKC(cudaMemset(c->W, 0, (size_t)P * c->w_stride * sizeof(double)));
+  CKC(cudaMemsetAsync(c->H, 0, (size_t)P * c->h_stride * sizeof(double), c->stream));
+  CKC(cudaMemsetAsync(c->W, 0, (size_t)P * c->w_stride * sizeof(double), c->stream));
   CKC(cudaMalloc(&c->TLi, (size_t)P * c->t_stride * bb));
   CKC(cudaMalloc(&c->TDi, (size_t)P * c->t_stride * bb));
   CKC(dmalloc(&c->gp, (size_t)P * K));
@@ -175,7 +177,7 @@ lslu_status create_common(lslu_ctx* c, const int64_t* rp, const int32_t* ci, con
   CKC(dmalloc(&c->st, P));
   CKC(cudaMallocHost((void**)&c->st_host, sizeof(DevState) * P));
   std::memset(c->st_host, 0, sizeof(DevState) * P);
-  CKC(cudaMemset(c->st, 0, sizeof(DevState) * P));
+  CKC(cudaMemsetAsync(c->st, 0, sizeof(DevState) * P, c->stream));
   c->pw_cluster = projected_cluster_size();
   // LSLU_NO_GRAPHS=1: launch every kernel directly instead of replaying
   // captured graphs (for kernel-level profilers)
@@ -1420,8 +1422,8 @@ extern "C" lslu_status lslu_set_loop(lslu_handle h, int32_t mode, int32_t blocks
     CK(dmalloc(&c->pq_keys, 2 * (size_t)c->nprob));
     CK(dmalloc(&c->pq_bar, 4));
     CK(dmalloc(&c->pq_err, 1));
-    CK(cudaMemset(c->pq_bar, 0, 4 * sizeof(unsigned)));
-    CK(cudaMemset(c->pq_err, 0, sizeof(int)));
+    CK(cudaMemsetAsync(c->pq_bar, 0, 4 * sizeof(unsigned), c->stream));
+    CK(cudaMemsetAsync(c->pq_err, 0, sizeof(int), c->stream));
     if (c->nprob > 1) {
       CK(dmalloc(&c->pq_row0, (size_t)c->nprob));
       CK(dmalloc(&c->pq_col0, (size_t)c->nprob));
