@@ -262,6 +262,20 @@ void check_csr_host(int64_t nnz, int64_t n, const int32_t* ci, const double* vv,
   }
 }
 
+// Whether kernels on the current device may read a caller's device array where
+// it is: aligned to its elements, and managed or on this device.  (A copy takes
+// any address of any device.)
+bool readable_in_place(const void* p, size_t align) {
+  if (reinterpret_cast<uintptr_t>(p) % align != 0) return false;
+  cudaPointerAttributes at;
+  int dev = 0;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev);
+}
+
 lslu_status create_single(int64_t m, int64_t n, int64_t nnz, const int64_t* row_ptr,
                           const int32_t* col_idx, const double* vals, int32_t value_type,
                           int32_t max_iter, const int32_t* row_order, const int32_t* col_order,
@@ -282,15 +296,30 @@ lslu_status create_single(int64_t m, int64_t n, int64_t nnz, const int64_t* row_
   if (!row_ptr || (nnz > 0 && (!col_idx || !vals)))
     return set_err(nullptr, LSLU_ERR_INVALID_ARG, "NULL CSR array");
 
-  // row pointers on the host; columns and values stay where they are
-  const bool on_device = ptr_location == LSLU_DEVICE;
+  // row pointers on the host; columns and values stay where they are if kernels
+  // can read them there, and come to the host otherwise
+  bool on_device = ptr_location == LSLU_DEVICE;
   std::vector<int64_t> rp_h;
+  std::vector<int32_t> ci_h;
+  std::vector<double> vv_h;
   if (on_device) {
     rp_h.resize(m + 1);
-    const cudaError_t e = cudaMemcpy(rp_h.data(), row_ptr, (m + 1) * 8, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess)
-      return set_err(nullptr, LSLU_ERR_CUDA, std::string("copying CSR: ") + cudaGetErrorString(e));
+    cudaError_t e = cudaMemcpy(rp_h.data(), row_ptr, (m + 1) * 8, cudaMemcpyDeviceToHost);
     row_ptr = rp_h.data();
+    if (e == cudaSuccess && nnz > 0 &&
+        !(readable_in_place(col_idx, sizeof(int32_t)) && readable_in_place(vals, sizeof(double)))) {
+      ci_h.resize(nnz);
+      vv_h.resize(nnz);
+      e = cudaMemcpy(ci_h.data(), col_idx, nnz * 4, cudaMemcpyDeviceToHost);
+      if (e == cudaSuccess) e = cudaMemcpy(vv_h.data(), vals, nnz * 8, cudaMemcpyDeviceToHost);
+      col_idx = ci_h.data();
+      vals = vv_h.data();
+      on_device = false;
+    }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      return set_err(nullptr, LSLU_ERR_CUDA, std::string("copying CSR: ") + cudaGetErrorString(e));
+    }
   }
   if (row_ptr[0] != 0 || row_ptr[m] != nnz)
     return set_err(nullptr, LSLU_ERR_INVALID_ARG, "row_ptr[0] must be 0 and row_ptr[m] == nnz");
