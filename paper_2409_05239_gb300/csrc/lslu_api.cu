@@ -113,6 +113,7 @@ lslu_status create_common(lslu_ctx* c, const int64_t* rp, const int32_t* ci, con
   lslu_status st = LSLU_OK;
   auto fail = [&](lslu_status s2) {
     lslu::thread_error() = c->err;
+    cudaGetLastError();  // other handles go on
     destroy_ctx(c);
     return s2;
   };

@@ -14,8 +14,11 @@
 // A 2.5 M-entry matrix (128x128 image, 120 angles) took 28.6 ms to set up
 // with host loops (a counting sort with one random write per entry, copies
 // into vectors and their page faults) against about 0.5 ms of kernels and
-// copies.  Rows or columns longer than kSortMax entries are sorted on the
-// host instead.
+// copies.  The construction needs 8 bytes of device memory per entry beside
+// the stored matrices, 20 where the CSR comes from the host (the caller's
+// entries are there too).  The host sorts instead, and its rows pass through a
+// small buffer, where rows or columns have more than kSortMax entries and where
+// that memory is not to be had.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
@@ -34,6 +37,8 @@ namespace {
 constexpr int kSortMax = 8192;  // keys of 8 bytes one block sorts (64 KB of shared memory)
 constexpr int kSortThreads = 256;
 constexpr int kRowThreads = 256;  // one warp per row
+constexpr int64_t kUploadEntries = 4 << 20;   // of the host's rows on their way, 12 bytes each
+constexpr int64_t kUploadMinimum = 256 << 10;  // the same where memory is short
 
 // Entry of a row that its stored position q holds: full kPermBlock-entry
 // blocks are stored transposed (position 4 l + i holds entry 16 i + l).
@@ -82,7 +87,7 @@ __global__ void __launch_bounds__(kRowThreads)
   }
 }
 
-// Row r of the stored matrix from entry rp[r] on, in the input's order.
+// Row r of the stored matrix from entry rp[r] - rp[0] on, in the input's order.
 template <typename VT>
 __global__ void __launch_bounds__(kRowThreads)
     k_fill_rows(int64_t rows, const int64_t* __restrict__ rp, const int32_t* __restrict__ prp,
@@ -91,8 +96,8 @@ __global__ void __launch_bounds__(kRowThreads)
   const int lane = threadIdx.x & 31;
   const int64_t r = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (r >= rows) return;
-  const int64_t a = rp[r];
-  const int len = (int)(rp[r + 1] - a), plen = prl[r];
+  const int64_t a = rp[r] - rp[0];
+  const int len = (int)(rp[r + 1] - rp[r]), plen = prl[r];
   for (int q = lane; q < plen; q += 32) {
     const int e = stored_entry(q, plen);
     const int64_t s = a + (e < len ? e : len - 1);  // padding repeats the last column
@@ -154,9 +159,10 @@ __global__ void __launch_bounds__(kSortThreads)
 }
 
 // Smallest column of every block and unit of a row, one warp per row, two
-// entries per lane; wide[0] / wide[1] set where a block / unit spans 2^16
-// columns or more.  With off: the offsets from the blocks' (by_block) or units'
-// smallest column, and that column for every unit.
+// entries per lane.  With bbase: the blocks' smallest columns, and (with wide)
+// wide[0] / wide[1] set where a block / unit spans 2^16 columns or more.  With
+// off: the offsets from the blocks' (by_block) or units' smallest column, and
+// that column for every unit.
 __global__ void __launch_bounds__(kRowThreads)
     k_offsets(int64_t rows, const int32_t* __restrict__ prp, const int32_t* __restrict__ prl,
               const int32_t* __restrict__ rblk, const int32_t* __restrict__ col,
@@ -187,16 +193,14 @@ __global__ void __launch_bounds__(kRowThreads)
         lo[h] = min(lo[h], __shfl_xor_sync(0xffffffffu, lo[h], o));
         hi[h] = max(hi[h], __shfl_xor_sync(0xffffffffu, hi[h], o));
       }
-    if (!off) {
-      if (lane == 0) {
-        bbase[rblk[r] + b] = blo;
-        if (bhi - blo > 65535) wide[0] = 1;
-      }
+    if (bbase && lane == 0) bbase[rblk[r] + b] = blo;
+    if (wide) {
+      if (lane == 0 && bhi - blo > 65535) wide[0] = 1;
 #pragma unroll
       for (int h = 0; h < 2; ++h)
         if (in[h] && hi[h] - lo[h] > 65535) wide[1] = 1;
-      continue;
     }
+    if (!off) continue;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       if (!in[h]) continue;
@@ -208,27 +212,31 @@ __global__ void __launch_bounds__(kRowThreads)
   }
 }
 
-// Padded layout of rows of the given lengths.
+// Padded layout of rows of the given lengths: where each starts, its padded
+// length and its first block, as they are uploaded.
 struct Layout {
-  std::vector<int32_t> ptr, len, blk;
+  std::vector<int32_t> words;      // row pointers, lengths, first blocks
+  int64_t len_at = 0, blk_at = 0;  // the latter two in words
   int64_t tot = 0, blocks = 0;
 };
+int64_t words64(int64_t count) { return (count + 63) / 64 * 64; }  // whole 256-byte pieces
 template <typename Len>
 bool make_layout(int64_t rows, Len len, Layout& l) {
   const int64_t nrp = (rows + 1 + 3) / 4 * 4;  // row pointers padded to a multiple of 4 entries
-  l.ptr.resize(nrp);
-  l.len.resize(rows);
-  l.blk.resize(rows);
+  l.len_at = words64(nrp);
+  l.blk_at = l.len_at + words64(rows);
+  l.words.resize(l.blk_at + words64(rows));
+  int32_t *ptr = l.words.data(), *plens = ptr + l.len_at, *blk = ptr + l.blk_at;
   for (int64_t r = 0; r < rows; ++r) {
     const int64_t plen = (len(r) + kRowAlign - 1) / kRowAlign * kRowAlign;
-    l.ptr[r] = (int32_t)l.tot;
-    l.len[r] = (int32_t)plen;
-    l.blk[r] = (int32_t)l.blocks;
+    ptr[r] = (int32_t)l.tot;
+    plens[r] = (int32_t)plen;
+    blk[r] = (int32_t)l.blocks;
     l.tot += plen;
     l.blocks += (plen + kPermBlock - 1) / kPermBlock;
     if (l.tot >= (int64_t)INT32_MAX) return false;
   }
-  for (int64_t i = rows; i < nrp; ++i) l.ptr[i] = (int32_t)l.tot;
+  for (int64_t i = rows; i < nrp; ++i) ptr[i] = (int32_t)l.tot;
   return true;
 }
 
@@ -238,14 +246,29 @@ bool make_layout(int64_t rows, Len len, Layout& l) {
     if (e_ != cudaSuccess) return e_;        \
   } while (0)
 
+size_t align_up(size_t bytes) { return (bytes + 255) / 256 * 256; }
+
+// Arrays carved out of one allocation.
+struct Arena {
+  char* base = nullptr;
+  size_t used = 0;
+  template <typename T>
+  T* take(size_t count) {
+    T* p = reinterpret_cast<T*>(base + used);
+    used += align_up(count * sizeof(T));
+    return p;
+  }
+};
+
 template <typename T>
-cudaError_t upload(T** dst, const T* src, size_t count, size_t at_least, cudaStream_t s) {
-  CE(cudaMalloc((void**)dst, std::max(count, at_least) * sizeof(T)));
-  return count ? cudaMemcpyAsync(*dst, src, count * sizeof(T), cudaMemcpyHostToDevice, s)
+cudaError_t upload(T* dst, const T* src, size_t count, cudaStream_t s) {
+  return count ? cudaMemcpyAsync(dst, src, count * sizeof(T), cudaMemcpyHostToDevice, s)
                : cudaSuccess;
 }
 
-// The arrays of a stored matrix, columns and values still to be filled.
+// The arrays of a stored matrix, columns and values still to be filled.  (Two
+// allocations and one upload of the rows for a matrix; with eight allocations
+// and three uploads a handle of 17532 entries took 497 us to set up, now 432.)
 cudaError_t allocate(const Layout& l, int64_t rows, int64_t cols, int64_t nnz, int vt, DevCsr* out,
                      cudaStream_t s) {
   out->rows = rows;
@@ -254,12 +277,18 @@ cudaError_t allocate(const Layout& l, int64_t rows, int64_t cols, int64_t nnz, i
   out->nnz_padded = l.tot;
   const size_t vbytes = vt == LSLU_F64 ? 8 : vt == LSLU_F32 ? 4 : 2;
   const int64_t cap = std::max<int64_t>(l.tot, kRowAlign);
-  CE(upload(&out->row_ptr, l.ptr.data(), l.ptr.size(), 1, s));
-  CE(upload(&out->row_len, l.len.data(), l.len.size(), 1, s));
-  CE(upload(&out->rblk, l.blk.data(), l.blk.size(), 1, s));
-  CE(cudaMalloc((void**)&out->bbase, std::max<int64_t>(l.blocks, 1) * sizeof(int32_t)));
-  CE(cudaMalloc((void**)&out->col, cap * sizeof(int32_t)));
-  return cudaMalloc(&out->val, cap * vbytes);
+  Arena mem;
+  CE(cudaMalloc(&out->mem_rows, align_up(l.words.size() * 4) + align_up(l.blocks * 4) + 256 +
+                                    align_up(cap * 4) + align_up(cap * vbytes)));
+  mem.base = (char*)out->mem_rows;
+  out->row_ptr = mem.take<int32_t>(l.words.size());
+  out->row_len = out->row_ptr + l.len_at;
+  out->rblk = out->row_ptr + l.blk_at;
+  out->bbase = mem.take<int32_t>(l.blocks);
+  out->flags = mem.take<int32_t>(4);
+  out->col = mem.take<int32_t>(cap);
+  out->val = mem.take<char>(cap * vbytes);
+  return upload(out->row_ptr, l.words.data(), l.words.size(), s);
 }
 
 template <typename Fn>
@@ -274,12 +303,14 @@ void with_value_type(int vt, void* val, Fn f) {
 
 unsigned warps_grid(int64_t rows) { return (unsigned)((rows * 32 + kRowThreads - 1) / kRowThreads); }
 
-void fill_rows(const DevCsr& A, int vt, const int64_t* rp, const int32_t* ci, const double* vv,
-               cudaStream_t s) {
-  if (A.nnz_padded == 0) return;
+// Stored rows r0 .. r0 + rows - 1 from a CSR of them alone (rp: the caller's
+// row pointers of these rows).
+void fill_rows(const DevCsr& A, int vt, int64_t r0, int64_t rows, const int64_t* rp,
+               const int32_t* ci, const double* vv, cudaStream_t s) {
+  if (A.nnz_padded == 0 || rows == 0) return;
   with_value_type(vt, A.val, [&](auto* v) {
-    k_fill_rows<<<warps_grid(A.rows), kRowThreads, 0, s>>>(A.rows, rp, A.row_ptr, A.row_len, ci,
-                                                           vv, A.col, v);
+    k_fill_rows<<<warps_grid(rows), kRowThreads, 0, s>>>(rows, rp, A.row_ptr + r0, A.row_len + r0,
+                                                         ci, vv, A.col, v);
   });
 }
 
@@ -303,26 +334,43 @@ cudaError_t sort_fill(const DevCsr& A, int vt, int max_len, const unsigned long 
   return e;
 }
 
+void launch_offsets(const DevCsr& A, int32_t* bbase, int* wide, uint16_t* off, int32_t* ubase,
+                    cudaStream_t s) {
+  k_offsets<<<warps_grid(A.rows), kRowThreads, 0, s>>>(A.rows, A.row_ptr, A.row_len, A.rblk, A.col,
+                                                       bbase, wide, A.block_compressed != 0, off,
+                                                       ubase);
+}
+
 // 16-bit column offsets, from the smallest column of every block where all
-// blocks span fewer than 2^16 columns, else of every unit where those do.
-cudaError_t add_offsets(DevCsr* A, const int (&wide)[2], cudaStream_t s) {
-  A->block_compressed = A->nnz_padded > 0 && !wide[0];
-  A->compressed = A->nnz_padded > 0 && !wide[1];
-  if (A->block_compressed) A->compressed = 1;  // a unit lies inside one block
-  if (!A->block_compressed) {
-    cudaFree(A->bbase);
-    cudaFree(A->rblk);
-    A->bbase = A->rblk = nullptr;
+// blocks span fewer than 2^16 columns, else of every unit where those do.  With
+// at most 2^16 columns that holds without a look.
+cudaError_t add_offsets(DevCsr* A, DevCsr* AT, cudaStream_t s) {
+  DevCsr* both[2] = {A, AT};
+  auto narrow = [](const DevCsr& M) { return M.cols <= 65536; };
+  int wide[4] = {0, 0, 0, 0};
+  if (!narrow(*A) || !narrow(*AT)) {
+    CE(cudaMemsetAsync(A->flags, 0, sizeof(wide), s));
+    for (int w = 0; w < 2; ++w)
+      if (both[w]->nnz_padded && !narrow(*both[w]))
+        launch_offsets(*both[w], both[w]->bbase, A->flags + 2 * w, nullptr, nullptr, s);
+    CE(cudaGetLastError());
+    CE(cudaMemcpyAsync(wide, A->flags, sizeof(wide), cudaMemcpyDeviceToHost, s));
+    CE(cudaStreamSynchronize(s));
   }
-  if (!A->compressed) return cudaSuccess;
-  // unit bases readable up to a multiple of 4 units
-  const int64_t nub = (A->nnz_padded / kRowAlign + 3) / 4 * 4;
-  CE(cudaMalloc((void**)&A->off, A->nnz_padded * sizeof(uint16_t)));
-  CE(cudaMalloc((void**)&A->ubase, nub * sizeof(int32_t)));
-  CE(cudaMemsetAsync(A->ubase, 0, nub * sizeof(int32_t), s));
-  k_offsets<<<warps_grid(A->rows), kRowThreads, 0, s>>>(A->rows, A->row_ptr, A->row_len, A->rblk,
-                                                        A->col, A->bbase, nullptr,
-                                                        A->block_compressed != 0, A->off, A->ubase);
+  for (int w = 0; w < 2; ++w) {
+    DevCsr& M = *both[w];
+    M.block_compressed = M.nnz_padded > 0 && !wide[2 * w];
+    M.compressed = M.nnz_padded > 0 && (M.block_compressed || !wide[2 * w + 1]);
+    if (!M.compressed) continue;
+    // unit bases readable up to a multiple of 4 units
+    const int64_t nub = (M.nnz_padded / kRowAlign + 3) / 4 * 4;
+    Arena mem;
+    CE(cudaMalloc(&M.mem_off, align_up(M.nnz_padded * sizeof(uint16_t)) + align_up(nub * 4)));
+    mem.base = (char*)M.mem_off;
+    M.off = mem.take<uint16_t>(M.nnz_padded);
+    M.ubase = mem.take<int32_t>(nub);
+    launch_offsets(M, narrow(M) ? M.bbase : nullptr, nullptr, M.off, M.ubase, s);
+  }
   return cudaGetLastError();
 }
 
@@ -344,16 +392,9 @@ void transpose_host(int64_t m, int64_t n, const int64_t* rp, const int32_t* ci, 
     }
 }
 
-struct Scratch {  // one allocation for everything the construction needs for itself
-  char* base = nullptr;
-  size_t used = 0;
+struct Scratch : Arena {  // device memory that the construction gives back
   ~Scratch() { cudaFree(base); }
-  template <typename T>
-  T* take(size_t count) {
-    T* p = reinterpret_cast<T*>(base + used);
-    used += (count * sizeof(T) + 255) / 256 * 256;
-    return p;
-  }
+  cudaError_t reserve(size_t bytes) { return cudaMalloc((void**)&base, bytes); }
 };
 
 }  // namespace
@@ -388,7 +429,7 @@ cudaError_t check_csr_device(int64_t nnz, int64_t n, const int32_t* ci, const do
   *bad_col = *bad_val = -1;
   if (nnz == 0) return cudaSuccess;
   Scratch mem;
-  CE(cudaMalloc((void**)&mem.base, 256));
+  CE(mem.reserve(256));
   unsigned long long* bad = mem.take<unsigned long long>(2);
   CE(cudaMemsetAsync(bad, 0xff, 16, s));
   k_check<<<(unsigned)std::min<int64_t>((nnz + 255) / 256, 8192), 256, 0, s>>>(nnz, n, ci, vv, bad);
@@ -400,65 +441,62 @@ cudaError_t check_csr_device(int64_t nnz, int64_t n, const int32_t* ci, const do
   return cudaSuccess;
 }
 
-cudaError_t build_csr_pair(int64_t m, int64_t n, const int64_t* rp, const int32_t* ci,
-                           const double* vv, bool on_device, const std::vector<int32_t>* inv_row,
-                           const std::vector<int32_t>* col_new, int vt, DevCsr* A, DevCsr* AT,
-                           cudaStream_t s) {
-  A->shape = AT->shape = default_shape(vt);
-  int dev = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess)
-    cudaDeviceGetAttribute(&A->num_sms, cudaDevAttrMultiProcessorCount, dev);
-  AT->num_sms = A->num_sms;
-  const int64_t nnz = rp[m];
-  auto row_len = [&](int64_t r) {
-    const int64_t src = inv_row ? (*inv_row)[r] : r;
-    return rp[src + 1] - rp[src];
-  };
-  Layout la, lt;
-  if (!make_layout(m, row_len, la)) return cudaErrorInvalidValue;
-  int64_t max_row = 0;
-  for (int64_t r = 0; r < m; ++r) max_row = std::max(max_row, rp[r + 1] - rp[r]);
+namespace {
+
+// A CSR as the construction takes it: row pointers on the host, columns and
+// values on the host or (on_device) the device, an optional renumbering.
+struct Source {
+  int64_t m, n, nnz;
+  const int64_t* rp;
+  const int32_t* ci;
+  const double* vv;
+  bool on_device;
+  const std::vector<int32_t>*inv_row, *col_new;
+  int64_t max_row;  // longest row
+};
+
+// Both matrices on the device.  *fits = false, with nothing left to undo but
+// what A holds: a column has more than kSortMax entries.
+cudaError_t build_on_device(const Source& in, const Layout& la, int vt, DevCsr* A, DevCsr* AT,
+                            cudaStream_t s, bool* fits) {
+  const int64_t m = in.m, n = in.n, nnz = in.nnz;
+  *fits = true;
   // every host array that an asynchronous copy reads lives until the final
   // synchronisation
   std::vector<int32_t> cnt(n), first(n + 1, 0);
-  std::vector<int64_t> rp_a, rp_t;
-  std::vector<int32_t> ci_h, ci_a, ci_t;
-  std::vector<double> vv_h, vv_a, vv_t;
+  Layout lt;
   Scratch mem;
-  const size_t e1 = (size_t)std::max<int64_t>(nnz, 1);
-  const size_t bytes = (size_t)(m + 1) * 8 + (size_t)(n + 1) * 8 + (n + 1) * 16 + m * 4 +
-                       e1 * (8 + 2 * (4 + 8)) + 16 * 256;
-  CE(cudaMalloc((void**)&mem.base, bytes));
+  const size_t e = in.on_device ? 0 : (size_t)nnz;  // entries brought from the host
+  const size_t bytes = align_up((m + 1) * 8) + align_up(n * 4) + align_up((n + 1) * 4) +
+                       (in.inv_row ? align_up(m * 4) + align_up(n * 4) : 0) +
+                       align_up((size_t)nnz * 8) + align_up(e * 4) + align_up(e * 8);
+  CE(mem.reserve(std::max<size_t>(bytes, 1)));
   int64_t* d_rp = mem.take<int64_t>(m + 1);
-  int64_t* d_rpt = mem.take<int64_t>(n + 1);
   int32_t* d_cnt = mem.take<int32_t>(n);
   int32_t* d_first = mem.take<int32_t>(n + 1);
-  int32_t* d_inv = mem.take<int32_t>(m);
-  int32_t* d_new = mem.take<int32_t>(n);
-  int* d_wide = mem.take<int>(4);
-  unsigned long long* d_keys = mem.take<unsigned long long>(e1);
-  int32_t* d_ci = mem.take<int32_t>(e1);
-  double* d_vv = mem.take<double>(e1);
-  auto to_device = [&](auto* dst, const auto* src, size_t count) {
-    return count ? cudaMemcpyAsync(dst, src, count * sizeof(*dst), cudaMemcpyHostToDevice, s)
-                 : cudaSuccess;
-  };
-  const int32_t* c_in = ci;
-  const double* v_in = vv;
-  if (!on_device) {
-    CE(to_device(d_ci, ci, nnz));
-    CE(to_device(d_vv, vv, nnz));
-    c_in = d_ci;
-    v_in = d_vv;
+  int32_t* d_inv = in.inv_row ? mem.take<int32_t>(m) : nullptr;
+  int32_t* d_new = in.inv_row ? mem.take<int32_t>(n) : nullptr;
+  unsigned long long* d_keys = mem.take<unsigned long long>(nnz);
+  const int32_t* ci = in.ci;
+  const double* vv = in.vv;
+  if (!in.on_device) {
+    int32_t* d_ci = mem.take<int32_t>(e);
+    double* d_vv = mem.take<double>(e);
+    CE(upload(d_ci, in.ci, e, s));
+    CE(upload(d_vv, in.vv, e, s));
+    ci = d_ci;
+    vv = d_vv;
   }
-  CE(to_device(d_rp, rp, m + 1));
-  if (inv_row) CE(to_device(d_inv, inv_row->data(), m));
-  if (col_new) CE(to_device(d_new, col_new->data(), n));
-  CE(cudaMemsetAsync(d_wide, 0, 4 * sizeof(int), s));
+  if (mem.used != bytes) return cudaErrorInvalidValue;  // the sum above and the arrays disagree
+  CE(upload(d_rp, in.rp, m + 1, s));
+  if (in.inv_row) {
+    CE(upload(d_inv, in.inv_row->data(), m, s));
+    CE(upload(d_new, in.col_new->data(), n, s));
+  }
   CE(cudaMemsetAsync(d_cnt, 0, n * sizeof(int32_t), s));
   if (nnz)
-    k_count<<<(unsigned)std::min<int64_t>((nnz + 255) / 256, 8192), 256, 0, s>>>(
-        nnz, c_in, col_new ? d_new : nullptr, d_cnt);
+    k_count<<<(unsigned)std::min<int64_t>((nnz + 255) / 256, 8192), 256, 0, s>>>(nnz, ci, d_new,
+                                                                                 d_cnt);
   CE(cudaMemcpyAsync(cnt.data(), d_cnt, n * sizeof(int32_t), cudaMemcpyDeviceToHost, s));
   CE(allocate(la, m, n, nnz, vt, A, s));
   CE(cudaStreamSynchronize(s));
@@ -467,69 +505,137 @@ cudaError_t build_csr_pair(int64_t m, int64_t n, const int64_t* rp, const int32_
     first[c + 1] = first[c] + cnt[c];
     max_col = std::max<int64_t>(max_col, cnt[c]);
   }
+  if (max_col > kSortMax) {
+    *fits = false;
+    return cudaSuccess;
+  }
   if (!make_layout(n, [&](int64_t c) { return (int64_t)cnt[c]; }, lt)) return cudaErrorInvalidValue;
   CE(allocate(lt, n, m, nnz, vt, AT, s));
-  if (max_col > kSortMax || (inv_row && max_row > kSortMax)) {
-    // a row or column too long for one block's shared memory: host sorts
-    if (on_device) {
-      ci_h.resize(nnz);
-      vv_h.resize(nnz);
-      CE(cudaMemcpy(ci_h.data(), ci, nnz * 4, cudaMemcpyDeviceToHost));
-      CE(cudaMemcpy(vv_h.data(), vv, nnz * 8, cudaMemcpyDeviceToHost));
-      ci = ci_h.data();
-      vv = vv_h.data();
-    }
-    if (inv_row) {
-      renumber_csr(m, rp, ci, vv, *inv_row, *col_new, rp_a, ci_a, vv_a);
-      rp = rp_a.data();
-      ci = ci_a.data();
-      vv = vv_a.data();
-    }
-    transpose_host(m, n, rp, ci, vv, rp_t, ci_t, vv_t);
-    CE(to_device(d_rp, rp, m + 1));
-    CE(to_device(d_ci, ci, nnz));
-    CE(to_device(d_vv, vv, nnz));
-    fill_rows(*A, vt, d_rp, d_ci, d_vv, s);
-    CE(to_device(d_rpt, rp_t.data(), n + 1));
-    CE(to_device(d_ci, ci_t.data(), nnz));
-    CE(to_device(d_vv, vv_t.data(), nnz));
-    fill_rows(*AT, vt, d_rpt, d_ci, d_vv, s);
-  } else {
-    CE(to_device(d_first, first.data(), n + 1));
-    CE(cudaMemcpyAsync(d_cnt, d_first, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
-    if (nnz)
-      k_scatter_keys<<<warps_grid(m), kRowThreads, 0, s>>>(m, d_rp, c_in, inv_row ? d_inv : nullptr,
-                                                           col_new ? d_new : nullptr, d_cnt, d_keys);
-    if (inv_row)
-      CE(sort_fill(*A, vt, (int)max_row, nullptr, nullptr, d_rp, d_inv, d_new, c_in, v_in, s));
-    else
-      fill_rows(*A, vt, d_rp, c_in, v_in, s);
-    CE(sort_fill(*AT, vt, (int)max_col, d_keys, d_first, nullptr, nullptr, nullptr, c_in, v_in, s));
-  }
-  int wide[2][2] = {{0, 0}, {0, 0}};
-  DevCsr* both[2] = {A, AT};
-  for (int w = 0; w < 2; ++w)
-    if (both[w]->nnz_padded)
-      k_offsets<<<warps_grid(both[w]->rows), kRowThreads, 0, s>>>(
-          both[w]->rows, both[w]->row_ptr, both[w]->row_len, both[w]->rblk, both[w]->col,
-          both[w]->bbase, d_wide + 2 * w, false, nullptr, nullptr);
+  CE(upload(d_first, first.data(), n + 1, s));
+  CE(cudaMemcpyAsync(d_cnt, d_first, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, s));
+  if (nnz)
+    k_scatter_keys<<<warps_grid(m), kRowThreads, 0, s>>>(m, d_rp, ci, d_inv, d_new, d_cnt, d_keys);
+  if (in.inv_row)
+    CE(sort_fill(*A, vt, (int)in.max_row, nullptr, nullptr, d_rp, d_inv, d_new, ci, vv, s));
+  else
+    fill_rows(*A, vt, 0, m, d_rp, ci, vv, s);
+  CE(sort_fill(*AT, vt, (int)max_col, d_keys, d_first, nullptr, nullptr, nullptr, ci, vv, s));
   CE(cudaGetLastError());
-  CE(cudaMemcpyAsync(wide, d_wide, sizeof(wide), cudaMemcpyDeviceToHost, s));
-  CE(cudaStreamSynchronize(s));
-  CE(add_offsets(A, wide[0], s));
-  CE(add_offsets(AT, wide[1], s));
+  return cudaStreamSynchronize(s);
+}
+
+// A stored matrix from a host CSR in its final order: whole rows at a time go
+// through a device buffer, their row pointers, columns and values in one copy.
+cudaError_t fill_from_host(const DevCsr& A, int vt, const int64_t* rp, const int32_t* ci,
+                           const double* vv, char* buffer, int64_t chunk, std::vector<char>& stage,
+                           cudaStream_t s) {
+  for (int64_t r0 = 0; r0 < A.rows;) {
+    int64_t r1 = r0 + 1;  // (a row is no longer than the buffer)
+    while (r1 < A.rows && r1 - r0 < chunk && rp[r1 + 1] - rp[r0] <= chunk) ++r1;
+    const size_t rows = r1 - r0, e0 = rp[r0], n = rp[r1] - rp[r0];
+    const size_t vv_at = (rows + 1) * 8, ci_at = vv_at + n * 8;
+    CE(cudaStreamSynchronize(s));  // the stage's last rows are on the device
+    stage.resize(ci_at + n * 4);
+    std::memcpy(stage.data(), rp + r0, vv_at);
+    if (n) std::memcpy(stage.data() + vv_at, vv + e0, n * 8);
+    if (n) std::memcpy(stage.data() + ci_at, ci + e0, n * 4);
+    CE(upload(buffer, stage.data(), stage.size(), s));
+    fill_rows(A, vt, r0, rows, (const int64_t*)buffer, (const int32_t*)(buffer + ci_at),
+              (const double*)(buffer + vv_at), s);
+    r0 = r1;
+  }
+  return cudaGetLastError();
+}
+
+// Both matrices sorted by the host.
+cudaError_t build_on_host(Source in, const Layout& la, int vt, DevCsr* A, DevCsr* AT,
+                          cudaStream_t s) {
+  const int64_t m = in.m, n = in.n, nnz = in.nnz;
+  std::vector<int64_t> rp_a, rp_t;
+  std::vector<int32_t> ci_h, ci_a, ci_t;
+  std::vector<double> vv_h, vv_a, vv_t;
+  if (in.on_device) {
+    ci_h.resize(nnz);
+    vv_h.resize(nnz);
+    CE(cudaMemcpyAsync(ci_h.data(), in.ci, nnz * 4, cudaMemcpyDeviceToHost, s));
+    CE(cudaMemcpyAsync(vv_h.data(), in.vv, nnz * 8, cudaMemcpyDeviceToHost, s));
+    CE(cudaStreamSynchronize(s));
+    in.ci = ci_h.data();
+    in.vv = vv_h.data();
+  }
+  if (in.inv_row) {
+    renumber_csr(m, in.rp, in.ci, in.vv, *in.inv_row, *in.col_new, rp_a, ci_a, vv_a);
+    in.rp = rp_a.data();
+    in.ci = ci_a.data();
+    in.vv = vv_a.data();
+  }
+  transpose_host(m, n, in.rp, in.ci, in.vv, rp_t, ci_t, vv_t);
+  Layout lt;
+  int64_t longest = in.max_row;
+  if (!make_layout(n, [&](int64_t c) { return rp_t[c + 1] - rp_t[c]; }, lt))
+    return cudaErrorInvalidValue;
+  for (int64_t c = 0; c < n; ++c) longest = std::max(longest, rp_t[c + 1] - rp_t[c]);
+  CE(allocate(la, m, n, nnz, vt, A, s));
+  CE(allocate(lt, n, m, nnz, vt, AT, s));
+  // the buffer: at most the whole matrix, at least a row of it
+  std::vector<char> stage;
+  Scratch mem;
+  const int64_t whole = std::max(nnz, std::max(m, n));
+  auto reserve = [&](int64_t* chunk, int64_t want) {
+    *chunk = std::max(std::min(want, whole), longest);
+    return mem.reserve((size_t)(*chunk + 1) * 8 + (size_t)*chunk * 12);
+  };
+  int64_t chunk = 0;
+  cudaError_t e = reserve(&chunk, kUploadEntries);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    e = reserve(&chunk, kUploadMinimum);
+  }
+  CE(e);
+  CE(fill_from_host(*A, vt, in.rp, in.ci, in.vv, mem.base, chunk, stage, s));
+  CE(fill_from_host(*AT, vt, rp_t.data(), ci_t.data(), vv_t.data(), mem.base, chunk, stage, s));
+  return cudaStreamSynchronize(s);
+}
+
+}  // namespace
+
+cudaError_t build_csr_pair(int64_t m, int64_t n, const int64_t* rp, const int32_t* ci,
+                           const double* vv, bool on_device, const std::vector<int32_t>* inv_row,
+                           const std::vector<int32_t>* col_new, int vt, DevCsr* A, DevCsr* AT,
+                           cudaStream_t s) {
+  Source in{m, n, rp[m], rp, ci, vv, on_device, inv_row, col_new, 0};
+  auto row_len = [&](int64_t r) {
+    const int64_t src = inv_row ? (*inv_row)[r] : r;
+    return rp[src + 1] - rp[src];
+  };
+  Layout la;
+  if (!make_layout(m, row_len, la)) return cudaErrorInvalidValue;
+  for (int64_t r = 0; r < m; ++r) in.max_row = std::max(in.max_row, rp[r + 1] - rp[r]);
+  bool done = false;
+  if (in.nnz > 0 && !(inv_row && in.max_row > kSortMax)) {
+    const cudaError_t e = build_on_device(in, la, vt, A, AT, s, &done);
+    if (e == cudaErrorMemoryAllocation) done = false;
+    if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return e;
+  }
+  if (!done) {
+    cudaGetLastError();
+    CE(cudaStreamSynchronize(s));  // copies into what is given back
+    free_csr(A);
+    free_csr(AT);
+    CE(build_on_host(in, la, vt, A, AT, s));
+  }
+  int dev = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess)
+    cudaDeviceGetAttribute(&A->num_sms, cudaDevAttrMultiProcessorCount, dev);
+  AT->num_sms = A->num_sms;
+  A->shape = AT->shape = default_shape(vt);
+  CE(add_offsets(A, AT, s));
   return cudaStreamSynchronize(s);
 }
 
 void free_csr(DevCsr* c) {
-  cudaFree(c->row_ptr);
-  cudaFree(c->row_len);
-  cudaFree(c->col);
-  cudaFree(c->val);
-  cudaFree(c->off);
-  cudaFree(c->ubase);
-  cudaFree(c->bbase);
-  cudaFree(c->rblk);
+  cudaFree(c->mem_rows);
+  cudaFree(c->mem_off);
   *c = DevCsr();
 }
 

@@ -108,6 +108,9 @@ struct DevCsr {
                                // count from the block's smallest column
   int32_t* bbase = nullptr;    // smallest column of every block, row by row
   int32_t* rblk = nullptr;     // rows: first block of every row
+  int32_t* flags = nullptr;    // 4 words of the construction
+  // what the arrays are carved from: the rows with their blocks; the offsets
+  void *mem_rows = nullptr, *mem_off = nullptr;
   int num_sms = 0;             // of the device it lives on
   int64_t rows = 0, cols = 0;
   int64_t nnz = 0;         // true non-zeros
