@@ -298,7 +298,7 @@ lslu_status create_single(int64_t m, int64_t n, int64_t nnz, const int64_t* row_
     return set_err(nullptr, LSLU_ERR_INVALID_ARG, "NULL CSR array");
 
   // row pointers on the host; columns and values stay where they are if kernels
-  // can read them there, and come to the host otherwise
+  // can read them there, and come to the host otherwise and for small matrices
   bool on_device = ptr_location == LSLU_DEVICE;
   std::vector<int64_t> rp_h;
   std::vector<int32_t> ci_h;
@@ -308,7 +308,8 @@ lslu_status create_single(int64_t m, int64_t n, int64_t nnz, const int64_t* row_
     cudaError_t e = cudaMemcpy(rp_h.data(), row_ptr, (m + 1) * 8, cudaMemcpyDeviceToHost);
     row_ptr = rp_h.data();
     if (e == cudaSuccess && nnz > 0 &&
-        !(readable_in_place(col_idx, sizeof(int32_t)) && readable_in_place(vals, sizeof(double)))) {
+        (nnz <= kHostEntries || !readable_in_place(col_idx, sizeof(int32_t)) ||
+         !readable_in_place(vals, sizeof(double)))) {
       ci_h.resize(nnz);
       vv_h.resize(nnz);
       e = cudaMemcpy(ci_h.data(), col_idx, nnz * 4, cudaMemcpyDeviceToHost);

@@ -17,8 +17,8 @@
 // copies.  The construction needs 8 bytes of device memory per entry beside
 // the stored matrices, 20 where the CSR comes from the host (the caller's
 // entries are there too).  The host sorts instead, and its rows pass through a
-// small buffer, where rows or columns have more than kSortMax entries and where
-// that memory is not to be had.
+// small buffer, where rows or columns have more than kSortMax entries, where
+// that memory is not to be had, and for matrices of at most kHostEntries.
 #include <cuda_runtime.h>
 #include <cuda_bf16.h>
 
@@ -612,7 +612,7 @@ cudaError_t build_csr_pair(int64_t m, int64_t n, const int64_t* rp, const int32_
   if (!make_layout(m, row_len, la)) return cudaErrorInvalidValue;
   for (int64_t r = 0; r < m; ++r) in.max_row = std::max(in.max_row, rp[r + 1] - rp[r]);
   bool done = false;
-  if (in.nnz > 0 && !(inv_row && in.max_row > kSortMax)) {
+  if (in.nnz > kHostEntries && !(inv_row && in.max_row > kSortMax)) {
     const cudaError_t e = build_on_device(in, la, vt, A, AT, s, &done);
     if (e == cudaErrorMemoryAllocation) done = false;
     if (e != cudaSuccess && e != cudaErrorMemoryAllocation) return e;

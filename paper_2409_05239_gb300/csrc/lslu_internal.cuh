@@ -97,6 +97,13 @@ inline bool shape_cmp(int sh) {
 // against 22.0 at 3.2 M; a 32x32 solve (0.05 M) 2.20 against 2.15 ms.
 constexpr int64_t kStreamMinEntries = 1 << 20;
 
+// Entries up to which the host builds a handle's stored matrices (lslu_build.cu),
+// from device arrays too: the construction on the device is a dozen launches
+// and copies whatever the size.  Host / device arrays, us: 1784 entries 380 /
+// 430 by the host, 440 / 575 on the device; 8128: 415 / 474 against 456 / 590;
+// 17532: 512 / 693 against 482 / 597.
+constexpr int64_t kHostEntries = 8192;
+
 struct DevCsr {
   int shape = kShapeG16U2;
   int compressed = 0;          // 16-bit column offsets available (off, ubase)
