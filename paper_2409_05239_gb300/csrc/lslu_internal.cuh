@@ -116,7 +116,7 @@ struct DevCsr {
   int32_t* bbase = nullptr;    // smallest column of every block, row by row
   int32_t* rblk = nullptr;     // rows: first block of every row
   int32_t* flags = nullptr;    // 4 words of the construction
-  // what the arrays are carved from: the rows with their blocks; the offsets
+  // what the arrays of the rows with their blocks, and of the offsets, are carved from
   void *mem_rows = nullptr, *mem_off = nullptr;
   int num_sms = 0;             // of the device it lives on
   int64_t rows = 0, cols = 0;
