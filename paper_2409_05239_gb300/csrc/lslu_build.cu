@@ -47,6 +47,12 @@ __device__ __forceinline__ int stored_entry(int q, int plen) {
   return b < plen / kPermBlock ? b * kPermBlock + 16 * (w & 3) + (w >> 2) : q;
 }
 
+// Where entry e of a row is stored (the inverse).
+__device__ __forceinline__ int stored_position(int e, int plen) {
+  const int b = e / kPermBlock, w = e % kPermBlock;
+  return b < plen / kPermBlock ? b * kPermBlock + 4 * (w & 15) + (w >> 4) : e;
+}
+
 __device__ __forceinline__ void put(double* p, double v) { *p = v; }
 __device__ __forceinline__ void put(float* p, double v) { *p = __double2float_rn(v); }
 // FP64 -> FP32 -> BF16, each to nearest even, on the bits
@@ -375,6 +381,63 @@ cudaError_t add_offsets(DevCsr* A, DevCsr* AT, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// Neighbouring entries of every 16th row: count[0] pairs of different columns,
+// count[1] those whose FP32 vector entries share a 32-byte sector.
+__global__ void __launch_bounds__(kRowThreads)
+    k_near(int64_t rows, const int32_t* __restrict__ prp, const int32_t* __restrict__ prl,
+           const int32_t* __restrict__ col, int* count) {
+  const int lane = threadIdx.x & 31;
+  const int64_t r = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 16;
+  if (r >= rows) return;
+  const int32_t* c = col + prp[r];
+  const int plen = prl[r];
+  int pairs = 0, near = 0;
+  for (int e = lane; e + 1 < plen; e += 32) {
+    const int32_t a = c[stored_position(e, plen)], b = c[stored_position(e + 1, plen)];
+    pairs += a != b;  // (the padding repeats a row's last column)
+    near += a != b && (a >> 3) == (b >> 3);
+  }
+  pairs = __reduce_add_sync(0xffffffffu, pairs);
+  near = __reduce_add_sync(0xffffffffu, near);
+  if (lane == 0) {
+    atomicAdd(count, pairs);
+    atomicAdd(count + 1, near);
+  }
+}
+
+// The form of the default FP32 / BF16 products, by the mean length of a row.
+// A row under 64 entries gives a lane one chunk at most: there is nothing for
+// more of them in flight, and the plain form's six blocks per SM beat the
+// stream form's four.  Up to 96 entries, and where a row's columns are
+// scattered (fewer than one neighbour in ten in the same sector, as in a random
+// matrix), the products wait for their gathers, and the offsets form does best.
+// Whole solves of 20 to 300 iterations, FP32 / BF16, time against the plain
+// form's (products A and A^T alone behave alike):
+//   entries per row (A / A^T)               offsets        stream
+//   8 / 12, random columns                  1.00 / 1.00    1.10 / 1.12
+//   30 / 30, banded                         1.11 / 0.99    1.11 / 1.21
+//   461 / 76, 512x512 CT, 60 angles         0.96 / 0.95    0.97 / 1.05
+//   200 / 333, random columns               0.96 / 0.95    1.07 / 1.08
+//   144 / 153, 160x160 CT, 120 angles       0.99 / 0.96    0.91 / 0.91
+//   461 / 458, 512x512 CT, 360 angles       0.88           0.85
+cudaError_t choose_form(DevCsr* A, int vt, cudaStream_t s) {
+  A->form = kFormPlain;
+  if (vt == LSLU_F64 || A->nnz_padded < kStreamMinEntries || !A->compressed) return cudaSuccess;
+  const int64_t mean = A->nnz_padded / A->rows;
+  if (mean < 64) return cudaSuccess;
+  A->form = kFormOffsets;
+  if (mean < 96) return cudaSuccess;
+  int count[2];
+  CE(cudaMemsetAsync(A->flags, 0, sizeof(count), s));
+  k_near<<<warps_grid((A->rows + 15) / 16), kRowThreads, 0, s>>>(A->rows, A->row_ptr, A->row_len,
+                                                                 A->col, A->flags);
+  CE(cudaGetLastError());
+  CE(cudaMemcpyAsync(count, A->flags, sizeof(count), cudaMemcpyDeviceToHost, s));
+  CE(cudaStreamSynchronize(s));
+  if ((int64_t)count[1] * 10 >= count[0]) A->form = kFormStream;
+  return cudaSuccess;
+}
+
 // The transpose of a host CSR, by a stable counting sort.
 void transpose_host(int64_t m, int64_t n, const int64_t* rp, const int32_t* ci, const double* vv,
                     std::vector<int64_t>& rpt, std::vector<int32_t>& cit, std::vector<double>& vt) {
@@ -631,6 +694,8 @@ cudaError_t build_csr_pair(int64_t m, int64_t n, const int64_t* rp, const int32_
   AT->num_sms = A->num_sms;
   A->shape = AT->shape = default_shape(vt);
   CE(add_offsets(A, AT, s));
+  CE(choose_form(A, vt, s));
+  CE(choose_form(AT, vt, s));
   return cudaStreamSynchronize(s);
 }
 

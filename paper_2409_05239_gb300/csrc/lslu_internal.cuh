@@ -89,12 +89,19 @@ inline bool shape_cmp(int sh) {
   return (sh >= kShapesPerFormat && sh < kShapeE8) || (sh >= kShapeE8 && (sh & 1));
 }
 
-// Entries (with padding) from which the default FP32 / BF16 products read
-// 16-bit offsets with four chunks in flight (stream_rows).  Below, the matrix
-// stays in L2 and a product is a few dependent round trips, where the extra
-// base read and the wider step cost more than the bytes: a pair of products
-// 8.2 us either way up to 0.4 M entries, 12.4 against 14.6 us at 1.35 M, 18.4
-// against 22.0 at 3.2 M; a 32x32 solve (0.05 M) 2.20 against 2.15 ms.
+// How the default FP32 / BF16 products read a matrix (chosen by choose_form;
+// the same sums, so the same bits):
+//   kFormPlain    32-bit columns, two chunks of a row in flight per lane;
+//   kFormOffsets  the same on 16-bit offsets;
+//   kFormStream   16-bit offsets, four chunks in flight, resident blocks that
+//                 take the row groups in turn (stream_rows).
+enum { kFormPlain = 0, kFormOffsets = 1, kFormStream = 2 };
+
+// Entries (with padding) from which they read 16-bit offsets.  Below, the
+// matrix stays in L2 and a product is a few dependent round trips, where the
+// extra base read and the wider step cost more than the bytes: a pair of
+// products 8.2 us either way up to 0.4 M entries, 12.4 against 14.6 us at
+// 1.35 M, 18.4 against 22.0 at 3.2 M; a 32x32 solve (0.05 M) 2.20 against 2.15 ms.
 constexpr int64_t kStreamMinEntries = 1 << 20;
 
 // Entries up to which the host builds a handle's stored matrices (lslu_build.cu),
@@ -116,6 +123,7 @@ struct DevCsr {
   int32_t* bbase = nullptr;    // smallest column of every block, row by row
   int32_t* rblk = nullptr;     // rows: first block of every row
   int32_t* flags = nullptr;    // 4 words of the construction
+  int form = kFormPlain;       // of the default FP32 / BF16 products
   // what the arrays of the rows with their blocks, and of the offsets, are carved from
   void *mem_rows = nullptr, *mem_off = nullptr;
   int num_sms = 0;             // of the device it lives on

@@ -214,6 +214,22 @@ bool native(int vt) {
   return (vt == LSLU_F64) == std::is_same<XT, double>::value;
 }
 
+// Calls f with a value of the FP32 / BF16 storage type and the chunks in
+// flight of the form (an integral_constant).
+template <typename Fn>
+void with_form(int form, int vt, Fn f) {
+  auto chunks = [&](auto v) {
+    if (form == kFormStream)
+      f(v, std::integral_constant<int, 4>{});
+    else
+      f(v, std::integral_constant<int, 2>{});
+  };
+  if (vt == LSLU_F32)
+    chunks(float{});
+  else
+    chunks(__nv_bfloat16{});
+}
+
 }  // namespace
 
 // Native products (FP64 vectors for FP64 values, FP32 otherwise) run in the
@@ -226,11 +242,10 @@ void launch_spmv(const DevCsr& A, int vt, const XT* x, YT* y, cudaStream_t s, in
     return;
   }
   if constexpr (std::is_same<XT, float>::value) {
-    if (A.nnz_padded >= kStreamMinEntries) {
-      if (vt == LSLU_F32)
-        spmv_run<float, XT, YT, 16, 4, true>(A, x, y, s);
-      else
-        spmv_run<__nv_bfloat16, XT, YT, 16, 4, true>(A, x, y, s);
+    if (A.form != kFormPlain) {
+      with_form(A.form, vt, [&](auto v, auto u) {
+        spmv_run<decltype(v), XT, YT, 16, decltype(u)::value, true>(A, x, y, s);
+      });
       return;
     }
   }
@@ -251,11 +266,10 @@ void launch_spmv_pivots(const DevCsr& A, int vt, const XT* x, YT* y, PivotCoef p
     return;
   }
   if constexpr (std::is_same<XT, float>::value) {
-    if (A.nnz_padded >= kStreamMinEntries) {
-      if (vt == LSLU_F32)
-        spmv_pivots_run<float, XT, YT, 16, 4, true>(A, x, y, pc, s);
-      else
-        spmv_pivots_run<__nv_bfloat16, XT, YT, 16, 4, true>(A, x, y, pc, s);
+    if (A.form != kFormPlain) {
+      with_form(A.form, vt, [&](auto v, auto u) {
+        spmv_pivots_run<decltype(v), XT, YT, 16, decltype(u)::value, true>(A, x, y, pc, s);
+      });
       return;
     }
   }

@@ -23,9 +23,9 @@
 namespace lslu {
 namespace {
 
-// The default FP32 / BF16 products run kStreamBlocksPerSm blocks per SM with
-// four chunks in flight per lane (64 registers) and hand every block several
-// row groups.  What bounds them is how many loads an SM keeps in flight: the
+// The stream form of the default FP32 / BF16 products runs kStreamBlocksPerSm
+// blocks per SM with four chunks in flight per lane (64 registers) and hands
+// every block several row groups.  What bounds them is how many loads an SM keeps in flight: the
 // matrix stream alone (no gathers) takes 113 us on the renumbered 512x512 CT
 // matrix (728 MB), a gather that always hits one L1 sector adds 15 us, its
 // real locality 4 us more.  Measured there, A / A^T in us (events around a
