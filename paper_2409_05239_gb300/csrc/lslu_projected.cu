@@ -700,7 +700,9 @@ __device__ __forceinline__ void warp_sum4(double (&v)[4], int lane) {
   for (int q = 0; q < 4; ++q) v[q] = __shfl_sync(0xffffffffu, c, 8 * q);
 }
 
-template <int NR, int NC, int CL>
+// TIMED: the time stamps of k_bidiag (the untimed form has no room in its
+// steps for them: 1% at k = 60).
+template <int NR, int NC, int CL, bool TIMED>
 __global__ void __launch_bounds__(kTB) k_bidiag_regs(ProjArgs a, ProjWork w) {
   constexpr int R = 32 * NR;       // rows held
   constexpr int NW = kTB / 32;     // warps per CTA
@@ -720,6 +722,10 @@ __global__ void __launch_bounds__(kTB) k_bidiag_regs(ProjArgs a, ProjWork w) {
   const Slots S = slot_of(w, pi);
   const double* Hp = a.H + (int64_t)pi.p * a.strideH;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  unsigned long long* ts =
+      TIMED && a.tstamp && pi.is_final && rank == 0 && tid == 0 ? a.tstamp : nullptr;
+  // (stored at the end: the words are in host memory)
+  const unsigned long long tbegin = TIMED && ts ? gtimer() : 0;
   const int v0 = rank + CL * warp;  // first column
   double m[NC][NR];                 // columns v0 + 4 CL i, rows lane + 32 e
 #pragma unroll
@@ -776,13 +782,23 @@ __global__ void __launch_bounds__(kTB) k_bidiag_regs(ProjArgs a, ProjWork w) {
     for (int r = (jn & ~31) + tid; r <= k; r += kTB)
       xP[jn & 1][r] = (part[0][r] + part[2][r]) + (part[1][r] + part[3][r]);
   };
+  unsigned long long tsec[4] = {0, 0, 0, 0}, tprev = TIMED && ts ? gtimer() : 0;
+  auto lap = [&](int q) {
+    if (TIMED && ts) {
+      const unsigned long long now = gtimer();
+      tsec[q] += now - tprev;
+      tprev = now;
+    }
+  };
   publish(0);
   for (int j = 0; j < k; ++j) {
     const int par = j & 1, e0 = (j + 1) >> 5;
+    lap(0);
     // Step j's vectors are complete in every CTA.  Those of parity par are
     // rewritten only in step j+2, after the next barrier, which no CTA passes
     // before all have read them below.
     cluster.sync();
+    lap(1);
     for (int r = (j & ~31) + tid / TPR; r <= (k | 31) && r < R; r += kTB / TPR) {
       constexpr int Q = CL / TPR;
       const int h = tid % TPR;  // TPR = 2: even and odd ranks
@@ -830,6 +846,7 @@ __global__ void __launch_bounds__(kTB) k_bidiag_regs(ProjArgs a, ProjWork w) {
       S.taur[j] = tr;
       S.Qs[(int64_t)j * k + j] = 1.0;
     }
+    lap(2);
     // own columns c > j: the right reflector, then the left one
     constexpr int NT = (NC + 3) / 4 * 4;
     double t[NT];
@@ -872,10 +889,17 @@ __global__ void __launch_bounds__(kTB) k_bidiag_regs(ProjArgs a, ProjWork w) {
           if (e >= e0) m[i][e] = fma(-h, u[e], m[i][e]);
       }
     }
+    lap(3);
     if (j + 1 < k) publish(j + 1);
   }
   // no CTA leaves while another may still read its shared memory
   cluster.sync();
+  if (TIMED && ts) {
+    const unsigned long long tend = gtimer();
+    ts[0] = tbegin;
+    ts[1] = tend;
+    for (int q = 0; q < 4; ++q) ts[8 + q] = tsec[q];
+  }
 }
 
 // ---- 2. singular values and weights ----------------------------------------
@@ -1814,8 +1838,10 @@ namespace {
 struct BidiagForm {
   int kmax, cluster;
   void (*kernel)(ProjArgs, ProjWork);
+  void (*timed)(ProjArgs, ProjWork);
 };
-const BidiagForm kBidiagForms[] = {{63, 8, k_bidiag_regs<2, 2, 8>}};
+const BidiagForm kBidiagForms[] = {
+    {63, 8, k_bidiag_regs<2, 2, 8, false>, k_bidiag_regs<2, 2, 8, true>}};
 }  // namespace
 
 // Per-device set-up of the projected kernels: their attributes (cluster size
@@ -1845,7 +1871,8 @@ ProjDeviceSetup setup_current_device() {
     d.num_sms = 0;
   cudaFuncSetAttribute(k_bidiag, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   for (const BidiagForm& f : kBidiagForms)
-    cudaFuncSetAttribute(f.kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    for (auto kernel : {f.kernel, f.timed})
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
   cudaFuncSetAttribute(k_bidiag, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap);
   cudaFuncSetAttribute(k_sigma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap);
   cudaFuncSetAttribute(k_sigma_lanes, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemCap);
@@ -1955,7 +1982,8 @@ cudaError_t launch_projected(const ProjArgs& a, ProjWork& w, cudaStream_t s, int
     const int count = batch ? nprob : hi - lo + 1;
     w.prob0 = batch ? 0 : lo - small;
     w.desc = !batch && count > 1;
-    const cudaError_t e = form ? launch_clusters(form->kernel, form->cluster, count, 0, a, w, s)
+    const cudaError_t e = form ? launch_clusters(a.tstamp ? form->timed : form->kernel, form->cluster,
+                                                      count, 0, a, w, s)
                                : launch_bidiag_general(a, w, hi, count, batch, dev_setup.num_sms, s);
     if (e != cudaSuccess) return e;
     ++launches;
