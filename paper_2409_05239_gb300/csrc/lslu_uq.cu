@@ -44,9 +44,9 @@ template <typename BT>
 constexpr bool kSkipOutside = sizeof(BT) == 8;
 
 // Row slices of one Gram tile: FP32 products are summed in FP32 within a slice
-// (64 slices at most); FP64 ones take as many as fill the GPU's FP64 pipes.
-template <typename BT>
-constexpr int kSlicesMax = sizeof(BT) == 8 ? 152 : 64;
+// (64 slices at most); FP64 ones take as many as fill the GPU's FP64 pipes, one
+// per SM.
+constexpr int kSlicesMaxF32 = 64;
 
 // Partial Gram tiles: block (pair, slice) adds B1(r, i) B2(r, j) over its rows
 // for the kTG x kTG tile (ti, tj) of the pair list; 256 threads, 4 x 4 outputs
@@ -417,17 +417,20 @@ lslu_status fail(Ctx* c, lslu_status st, const std::string& msg) {
 template <typename BT>
 cudaError_t gram(const BT* B1, int cols1, const BT* B2, int cols2, int64_t ld, int64_t rows,
                  bool symmetric, double* C, int64_t ldc, int2* dpairs, double* part,
-                 int64_t part_cap, cudaStream_t s) {
+                 int64_t part_cap, int num_sms, cudaStream_t s) {
   const int t1 = (cols1 + kTG - 1) / kTG, t2 = (cols2 + kTG - 1) / kTG;
   std::vector<int2> pairs;
   for (int i = 0; i < t1; ++i)
     for (int j = symmetric ? i : 0; j < t2; ++j) pairs.push_back(make_int2(i, j));
   const int np = (int)pairs.size();
-  int nsl = std::max(1, std::min(kSlicesMax<BT>, (960 + np - 1) / np));
+  int nsl = std::max(1, std::min(sizeof(BT) == 8 ? num_sms : kSlicesMaxF32, (960 + np - 1) / np));
   while (nsl > 1 && (int64_t)nsl * np * kTG * kTG > part_cap) --nsl;
   if ((int64_t)nsl * np * kTG * kTG > part_cap) return cudaErrorInvalidValue;
   int64_t rps = (rows + nsl - 1) / nsl;
   rps = (rps + kRC - 1) / kRC * kRC;
+  // slices past the rows would add zeros (900 x 576 FP64 bases, k = 40: 590 us
+  // a call with them, 549 without)
+  nsl = (int)((rows + rps - 1) / rps);
   cudaError_t e = cudaMemcpyAsync(dpairs, pairs.data(), np * sizeof(int2), cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return e;
   k_gram_tiles<BT><<<dim3(np, nsl), 256, 0, s>>>(B1, cols1, B2, cols2, ld, rows, dpairs, (int)rps,
@@ -497,9 +500,9 @@ lslu_status uq_impl(Ctx* c, double sigma2, double lam, double* var_diag, double*
   k_fill<BT><<<g, 256, 0, s>>>(ones, n, (BT)1);
   const double scale = sigma2 / (lam * lam);
   // Gram products
-  if ((e = gram<BT>(L, k, L, k, c->ldl, n, true, GL, k, pairs, part, part_cap, s)) != cudaSuccess ||
-      (e = gram<BT>(D, k, D, k, c->ldd, m, true, GD, k, pairs, part, part_cap, s)) != cudaSuccess ||
-      (e = gram<BT>(L, k, ones, 1, c->ldl, n, false, sL, k, pairs, part, part_cap, s)) !=
+  if ((e = gram<BT>(L, k, L, k, c->ldl, n, true, GL, k, pairs, part, part_cap, c->num_sms, s)) != cudaSuccess ||
+      (e = gram<BT>(D, k, D, k, c->ldd, m, true, GD, k, pairs, part, part_cap, c->num_sms, s)) != cudaSuccess ||
+      (e = gram<BT>(L, k, ones, 1, c->ldl, n, false, sL, k, pairs, part, part_cap, c->num_sms, s)) !=
           cudaSuccess) {
     cudaFree(base);
     return fail(c, LSLU_ERR_CUDA, std::string("uq gram: ") + cudaGetErrorString(e));
@@ -571,8 +574,8 @@ lslu_status gram_products_impl(Ctx* c, int k, const double* v, double* G, double
   if (e == cudaSuccess) {
     k_to_basis<BT><<<64, 256, 0, s>>>(v, vb, c->n);
     const BT* L = reinterpret_cast<const BT*>(c->L);
-    e = gram<BT>(L, k, L, k, c->ldl, c->n, true, G, k, pairs, part, part_cap, s);
-    if (e == cudaSuccess) e = gram<BT>(L, k, vb, 1, c->ldl, c->n, false, g, k, pairs, part, part_cap, s);
+    e = gram<BT>(L, k, L, k, c->ldl, c->n, true, G, k, pairs, part, part_cap, c->num_sms, s);
+    if (e == cudaSuccess) e = gram<BT>(L, k, vb, 1, c->ldl, c->n, false, g, k, pairs, part, part_cap, c->num_sms, s);
   }
   cudaFree(pairs);
   cudaFree(part);
