@@ -174,13 +174,27 @@ def spmv_bytes(P, value_type, cmp_A=False, cmp_AT=False):
     return 0.5 * (a + at)
 
 
-def stored_columns(shape, value_type):
-    """The column storage that a row shape reads, as spmv_bytes takes it.  The
-    default shape reads block offsets wherever every 64-entry block of the
-    matrix fits in 16 bits (as on the tomography matrices here)."""
-    if shape == ("16x1" if value_type == "f64" else "16x2"):
-        return "block"
-    return "16-bit" in shape
+def stored_columns(shape, value_type, row_lengths):
+    """The column storage that a row shape reads on a matrix with rows of these
+    lengths, as spmv_bytes takes it.  The default FP32 / BF16 shape reads 16-bit
+    offsets from 2^20 stored entries (rows padded to 8) and 64 per row on, and
+    counts them from block bases, since every 64-entry block of the tomography
+    matrices here spans fewer than 2^16 columns; the default FP64 shape reads
+    32-bit columns."""
+    if "16-bit" in shape:
+        return True
+    lengths = np.asarray(row_lengths, dtype=np.int64)
+    stored = int(((lengths + 7) // 8 * 8).sum())
+    offsets = shape == "16x2" and value_type != "f64" and stored >= 1 << 20 and \
+        stored // len(lengths) >= 64
+    return "block" if offsets else False
+
+
+def matrix_columns(Ps, value_type, shape_A, shape_AT):
+    """stored_columns of A and A^T of one problem or of a batch's stacked problems."""
+    A = np.concatenate([np.diff(P.row_ptr) for P in Ps])
+    AT = np.concatenate([np.bincount(P.col_idx, minlength=P.n) for P in Ps])
+    return stored_columns(shape_A, value_type, A), stored_columns(shape_AT, value_type, AT)
 
 
 def solve_bytes(P, value_type, K, cmp_A=False, cmp_AT=False):
@@ -526,7 +540,8 @@ def batched_study(dev, K=150, count=64, order="tiles", shape=None):
     for P in Ps:
         errs.append(np.linalg.norm(x[off:off + P.n] - P.x_true) / np.linalg.norm(P.x_true))
         off += P.n
-    nbytes = sum(solve_bytes(P, "f32", K, "block", "block") for P in Ps)
+    cols = matrix_columns(Ps, "f32", *[shape if all(shaped) and shape else "16x2"] * 2)
+    nbytes = sum(solve_bytes(P, "f32", K, *cols) for P in Ps)
     return {"problems": count, "K": K, "m_total": int(sum(P.m for P in Ps)),
             "n_total": int(sum(P.n for P in Ps)), "nnz_total": int(sum(P.nnz for P in Ps)),
             "numbering": ORDER_NOTE[order],
@@ -999,8 +1014,8 @@ def run_gpu(args):
         x = x_dev.cpu().numpy()
         rel_true = float(np.linalg.norm(x - P.x_true) / np.linalg.norm(P.x_true))
         cfg_sp = solver.spmv_config()
-        cmp_A = stored_columns(cfg_sp["shape_A"], args.value_type)
-        cmp_AT = stored_columns(cfg_sp["shape_AT"], args.value_type)
+        cmp_A, cmp_AT = matrix_columns([P], args.value_type, cfg_sp["shape_A"],
+                                       cfg_sp["shape_AT"])
         sbytes = spmv_bytes(P, args.value_type, cmp_A, cmp_AT)
         peaks = {}
         try:
