@@ -274,9 +274,7 @@ cudaError_t upload(T* dst, const T* src, size_t count, cudaStream_t s) {
 
 // The arrays of a stored matrix, columns and values still to be filled.  (Few
 // allocations and one upload of the rows: with eight allocations and three
-// uploads a handle of 17532 entries took 497 us to set up, now 440.  Columns
-// and values keep allocations of their own: where all shared one, a solve of a
-// 32 x 32 image with histories took 1610 instead of 1538 us.)
+// uploads a handle of 17532 entries took 497 us to set up, now 440.)
 cudaError_t allocate(const Layout& l, int64_t rows, int64_t cols, int64_t nnz, int vt, DevCsr* out,
                      cudaStream_t s) {
   out->rows = rows;
