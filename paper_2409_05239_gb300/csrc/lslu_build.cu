@@ -39,6 +39,7 @@ constexpr int kSortThreads = 256;
 constexpr int kRowThreads = 256;  // one warp per row
 constexpr int64_t kUploadEntries = 4 << 20;   // of the host's rows on their way, 12 bytes each
 constexpr int64_t kUploadMinimum = 256 << 10;  // the same where memory is short
+constexpr size_t kStageBytes = 512 << 10;       // rows put together for one copy
 
 // Entry of a row that its stored position q holds: full kPermBlock-entry
 // blocks are stored transposed (position 4 l + i holds entry 16 i + l).
@@ -587,7 +588,7 @@ cudaError_t build_on_device(const Source& in, const Layout& la, int vt, DevCsr* 
 }
 
 // A stored matrix from a host CSR in its final order: whole rows at a time go
-// through a device buffer, their row pointers, columns and values in one copy.
+// through a device buffer; of small matrices in one copy, put together in stage.
 cudaError_t fill_from_host(const DevCsr& A, int vt, const int64_t* rp, const int32_t* ci,
                            const double* vv, char* buffer, int64_t chunk, std::vector<char>& stage,
                            cudaStream_t s) {
@@ -595,13 +596,19 @@ cudaError_t fill_from_host(const DevCsr& A, int vt, const int64_t* rp, const int
     int64_t r1 = r0 + 1;  // (a row is no longer than the buffer)
     while (r1 < A.rows && r1 - r0 < chunk && rp[r1 + 1] - rp[r0] <= chunk) ++r1;
     const size_t rows = r1 - r0, e0 = rp[r0], n = rp[r1] - rp[r0];
-    const size_t vv_at = (rows + 1) * 8, ci_at = vv_at + n * 8;
-    CE(cudaStreamSynchronize(s));  // the stage's last rows are on the device
-    stage.resize(ci_at + n * 4);
-    std::memcpy(stage.data(), rp + r0, vv_at);
-    if (n) std::memcpy(stage.data() + vv_at, vv + e0, n * 8);
-    if (n) std::memcpy(stage.data() + ci_at, ci + e0, n * 4);
-    CE(upload(buffer, stage.data(), stage.size(), s));
+    const size_t vv_at = (rows + 1) * 8, ci_at = vv_at + n * 8, bytes = ci_at + n * 4;
+    if (bytes <= kStageBytes) {
+      CE(cudaStreamSynchronize(s));  // the stage's last rows are on the device
+      stage.resize(bytes);
+      std::memcpy(stage.data(), rp + r0, vv_at);
+      if (n) std::memcpy(stage.data() + vv_at, vv + e0, n * 8);
+      if (n) std::memcpy(stage.data() + ci_at, ci + e0, n * 4);
+      CE(upload(buffer, stage.data(), bytes, s));
+    } else {
+      CE(upload((int64_t*)buffer, rp + r0, rows + 1, s));
+      CE(upload((double*)(buffer + vv_at), vv + e0, n, s));
+      CE(upload((int32_t*)(buffer + ci_at), ci + e0, n, s));
+    }
     fill_rows(A, vt, r0, rows, (const int64_t*)buffer, (const int32_t*)(buffer + ci_at),
               (const double*)(buffer + vv_at), s);
     r0 = r1;
