@@ -362,8 +362,8 @@ __global__ void __launch_bounds__(kPT)
                     const DevState* st, const double* lam_ptr, const double* ybar, double* Mg,
                     double* zt_out, double* Hbar, double* scal, int in_smem) {
   // M and ztil in shared memory where they fit: every column of the factor
-  // waits for the one before, and in global memory each of those steps took
-  // several L2 round trips
+  // waits for the one before (a 900 x 576 gradient step of 120 iterations:
+  // 10.29 ms, 10.36 with M in global memory; no difference at K = 12)
   extern __shared__ double msh[];
   __shared__ double red[kPT / 32];
   __shared__ int bad;

@@ -1,5 +1,5 @@
 """The reflectors' FP64 reciprocal against exact values and CUDA's division, over the
-arguments that a reflector hands it (2^-480 .. 2^482) and beyond: one Halley step from an
+arguments that a reflector hands it (2^-480 .. 2^482) and beyond: one step of Chebyshev's method from an
 approximation of 2^-20 leaves at most 0.51 units of the last place, so a value differs from
 the correctly rounded one by a unit at most.  And the projected solve on H scaled by powers
 of two, up to and past the squares from which the reflectors divide instead (2^-959 and
