@@ -177,17 +177,20 @@ def spmv_bytes(P, value_type, cmp_A=False, cmp_AT=False):
 def stored_columns(shape, value_type, row_lengths):
     """The column storage that a row shape reads on a matrix with rows of these
     lengths, as spmv_bytes takes it.  The default FP32 / BF16 shape reads 16-bit
-    offsets from 2^20 stored entries (rows padded to 8) and 64 per row on, and
-    counts them from block bases, since every 64-entry block of the tomography
-    matrices here spans fewer than 2^16 columns; the default FP64 shape reads
-    32-bit columns."""
+    offsets from 2^20 stored entries (rows padded to 8) on, unless the rows are
+    many and short (more than three waves of 152 x 6 blocks of 16 rows, fewer
+    than 64 entries per row), and counts them from block bases, since every
+    64-entry block of the tomography matrices here spans fewer than 2^16 columns
+    and no row is far longer than the others; the default FP64 shape reads 32-bit
+    columns."""
     if "16-bit" in shape:
         return True
     lengths = np.asarray(row_lengths, dtype=np.int64)
     stored = int(((lengths + 7) // 8 * 8).sum())
-    offsets = shape == "16x2" and value_type != "f64" and stored >= 1 << 20 and \
-        stored // len(lengths) >= 64
-    return "block" if offsets else False
+    if shape != "16x2" or value_type == "f64" or stored < 1 << 20:
+        return False
+    few_rows = (len(lengths) + 15) // 16 <= 3 * 152 * 6
+    return "block" if few_rows or stored // len(lengths) >= 64 else False
 
 
 def matrix_columns(Ps, value_type, shape_A, shape_AT):

@@ -393,9 +393,9 @@ lslu_status lslu_uq(lslu_handle h, double sigma2, double lambda, int32_t ptr_loc
 
 /* Row shape of the sparse products: lanes per CSR row x chunks in flight per
  * lane.  Shapes 0-5 take chunks of 4 entries with 32-bit column indices (shape 0
- * on FP32/BF16 matrices with 2^20 entries and 64 per row or more reads the same
- * chunks through 16-bit offsets where the matrix has them, two or four in
- * flight: the same bits from fewer bytes):
+ * on most FP32/BF16 matrices from 2^20 entries on reads the same chunks through
+ * 16-bit offsets where the matrix has them, two or four in flight: the same bits
+ * from fewer bytes):
  * 0: 16x2 (default for FP32/BF16 values), 1: 32x1, 2: 16x1 (default for
  * FP64 values), 3: 8x1, 4: 8x2, 5: 4x1; shapes 6-11 are the same lane shapes
  * on 16-bit column offsets in chunks of 8 entries (2.5 instead of 4 bytes per

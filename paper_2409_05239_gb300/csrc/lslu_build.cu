@@ -225,6 +225,7 @@ struct Layout {
   std::vector<int32_t> words;      // row pointers, lengths, first blocks
   int64_t len_at = 0, blk_at = 0;  // the latter two in words
   int64_t tot = 0, blocks = 0;
+  int32_t max_len = 0;
 };
 int64_t words64(int64_t count) { return (count + 63) / 64 * 64; }  // whole 256-byte pieces
 template <typename Len>
@@ -240,6 +241,7 @@ bool make_layout(int64_t rows, Len len, Layout& l) {
     plens[r] = (int32_t)plen;
     blk[r] = (int32_t)l.blocks;
     l.tot += plen;
+    l.max_len = std::max(l.max_len, (int32_t)plen);
     l.blocks += (plen + kPermBlock - 1) / kPermBlock;
     if (l.tot >= (int64_t)INT32_MAX) return false;
   }
@@ -282,6 +284,7 @@ cudaError_t allocate(const Layout& l, int64_t rows, int64_t cols, int64_t nnz, i
   out->cols = cols;
   out->nnz = nnz;
   out->nnz_padded = l.tot;
+  out->max_len = l.max_len;
   const size_t vbytes = vt == LSLU_F64 ? 8 : vt == LSLU_F32 ? 4 : 2;
   const int64_t cap = std::max<int64_t>(l.tot, kRowAlign);
   Arena mem;
@@ -404,14 +407,13 @@ __global__ void __launch_bounds__(kRowThreads)
   }
 }
 
-// The form of the default FP32 / BF16 products, by the mean length of a row.
-// A row under 64 entries gives a lane one chunk at most: there is nothing for
-// more of them in flight, and the plain form's six blocks per SM beat the
-// stream form's four.  Up to 96 entries, and where a row's columns are
-// scattered (fewer than one neighbour in ten in the same sector, as in a random
-// matrix), the products wait for their gathers, and the offsets form does best.
-// Whole solves of 20 to 300 iterations, FP32 / BF16, time against the plain
-// form's (products A and A^T alone behave alike):
+// The form of the default FP32 / BF16 products.  A row under 64 entries gives a
+// lane one chunk at most: there is nothing for more of them in flight, and the
+// plain form's six blocks per SM beat the stream form's four.  Up to 96 entries,
+// and where a row's columns are scattered (fewer than one neighbour in ten in
+// the same sector, as in a random matrix), the products wait for their gathers,
+// and the offsets form does best.  Whole solves of 20 to 300 iterations, FP32 /
+// BF16, time against the plain form's (products A and A^T alone behave alike):
 //   entries per row (A / A^T)               offsets        stream
 //   8 / 12, random columns                  1.00 / 1.00    1.10 / 1.12
 //   30 / 30, banded                         1.11 / 0.99    1.11 / 1.21
@@ -419,12 +421,22 @@ __global__ void __launch_bounds__(kRowThreads)
 //   200 / 333, random columns               0.96 / 0.95    1.07 / 1.08
 //   144 / 153, 160x160 CT, 120 angles       0.99 / 0.96    0.91 / 0.91
 //   461 / 458, 512x512 CT, 360 angles       0.88           0.85
+// Two kinds of matrix take the stream form whatever their mean length.  A few
+// waves of row groups: resident blocks have no last wave, 40000 random rows of
+// 60 entries 0.96 / 0.97, 30000 banded ones of 80 0.87 / 0.87 (the table's first
+// rows have 300000 rows).  And a row far longer than a row group's share of the
+// matrix, a chain of its own that the product waits for: a banded matrix with 24
+// entries per row and a column of some 35000 takes 4.54 ms in place of 5.37.
 cudaError_t choose_form(DevCsr* A, int vt, cudaStream_t s) {
   A->form = kFormPlain;
   if (vt == LSLU_F64 || A->nnz_padded < kStreamMinEntries || !A->compressed) return cudaSuccess;
+  const int64_t groups = (A->rows + 15) / 16;                      // of 16 rows, one block's
+  const int64_t slots = std::max<int64_t>(A->num_sms * 6, 1);      // blocks of the plain form
+  const int64_t share = A->nnz_padded / (slots * 16);              // entries of a row group
   const int64_t mean = A->nnz_padded / A->rows;
-  if (mean < 64) return cudaSuccess;
-  A->form = kFormOffsets;
+  A->form = kFormStream;
+  if (groups <= 3 * slots || (A->max_len >= 1024 && A->max_len > 4 * share)) return cudaSuccess;
+  A->form = mean < 64 ? kFormPlain : kFormOffsets;
   if (mean < 96) return cudaSuccess;
   int count[2];
   CE(cudaMemsetAsync(A->flags, 0, sizeof(count), s));

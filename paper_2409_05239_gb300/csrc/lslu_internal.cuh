@@ -124,6 +124,7 @@ struct DevCsr {
   int32_t* rblk = nullptr;     // rows: first block of every row
   int32_t* flags = nullptr;    // 4 words of the construction
   int form = kFormPlain;       // of the default FP32 / BF16 products
+  int32_t max_len = 0;         // longest row (padded)
   // what the arrays of the rows with their blocks, and of the offsets, are carved from
   void *mem_rows = nullptr, *mem_off = nullptr;
   int num_sms = 0;             // of the device it lives on

@@ -18,8 +18,9 @@ import bench  # noqa: E402
     ("16x1/16-bit", "f64", 10, 3, True),
     # below 2^20 stored entries: 4681 rows of 217 entries, stored as 224, are above
     ("16x2", "f32", 4681, 224, False), ("16x2", "f32", 4682, 217, "block"),
-    # fewer than 64 stored entries per row
-    ("16x2", "f32", 30000, 56, False), ("16x2", "f32", 30000, 57, "block")])
+    # fewer than 64 stored entries per row, and more than 43776 rows
+    ("16x2", "f32", 43777, 56, False), ("16x2", "f32", 43777, 57, "block"),
+    ("16x2", "f32", 43776, 56, "block"), ("16x2", "f32", 30000, 40, "block")])
 def test_stored_columns(shape, value_type, rows, length, expect):
     assert bench.stored_columns(shape, value_type, np.full(rows, length)) == expect
 
@@ -36,9 +37,9 @@ def test_block_bytes_by_hand():
 def test_both_directions_of_a_batch():
     rng = np.random.default_rng(0)
     Ps = []
-    for m, n, L in ((6000, 12000, 100), (7000, 15000, 100)):
+    for m, n, L in ((6000, 22000, 100), (7000, 22000, 100)):
         Ps.append(types.SimpleNamespace(m=m, n=n, row_ptr=np.arange(m + 1) * L,
                                         col_idx=rng.integers(0, n, m * L)))
-    # rows of 104 stored entries; columns of about 50
+    # rows of 104 stored entries; 44000 columns of about 30
     assert bench.matrix_columns(Ps, "f32", "16x2", "16x2") == ("block", False)
     assert bench.matrix_columns(Ps[:1], "f32", "16x2", "16x2") == (False, False)

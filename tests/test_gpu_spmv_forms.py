@@ -1,9 +1,11 @@
 """The default FP32 / BF16 products of matrices from 2^20 entries on, over the forms that
-the mean row length and the neighbourhood of a row's columns choose (32-bit columns, 16-bit
+rows, row lengths and the neighbourhood of a row's columns choose (32-bit columns, 16-bit
 offsets, resident blocks) and the bases the offsets count from (blocks of 64 entries, units
 of 8): the column format is worked out here from the stored layout, every product must have
 the bits of the 32-bit path (a slice of the rows, too small for the others), and the
 products that several right-hand sides share the bits of the single ones."""
+import functools
+
 import numpy as np
 import pytest
 import scipy.sparse as sp
@@ -20,62 +22,70 @@ def built():
     build.build()
 
 
-def matrix(kind, mean, seed=1):
-    """CSR with rows of mean/2 .. 3 mean/2 sorted, distinct columns: neighbours in pairs
-    (2 columns, then a gap), evenly spread, or anywhere."""
-    rng = np.random.default_rng(seed)
-    m = 1_300_000 // mean
-    lens = rng.integers(mean // 2, mean + mean // 2 + 1, m)
+FEW, MANY = 4400, 46_000  # rows: below and above three waves of 912 blocks of 16
+
+
+@functools.lru_cache(maxsize=1)
+def matrix(kind, mean, rows, longest=0):
+    """CSR with rows of mean/2 .. 3 mean/2 sorted columns: neighbours in pairs (2 columns,
+    then a gap), evenly spread, or anywhere; one row of `longest` entries."""
+    rng = np.random.default_rng(1)
+    lens = rng.integers(mean // 2, mean + mean // 2 + 1, rows)
     lens[:3] = lens[-3:] = 0
-    spacing, n = {"pairs": (16, 20_000), "pairs wide": (2400, 1_000_000), "even": (8, 20_000),
+    lens[rows // 3] = longest or mean
+    ptr = np.zeros(rows + 1, np.int64)
+    np.cumsum(lens, out=ptr[1:])
+    row = np.repeat(np.arange(rows), lens)
+    e = np.arange(ptr[-1]) - ptr[row]
+    spacing, n = {"pairs": (16, 60_000), "pairs wide": (2400, 1_000_000), "even": (8, 60_000),
                   "even wide": (1200, 1_000_000), "anywhere": (None, 60_000),
                   "anywhere wide": (None, 6_000_000)}[kind]
-    rows = []
-    for L in lens:
-        if spacing is None:
-            rows.append(np.sort(rng.choice(n, L, replace=False)) if L else np.zeros(0, int))
-            continue
-        e = np.arange(L)
-        c = e // 2 * spacing + e % 2 if kind.startswith("pairs") else e * spacing
-        rows.append(c + 8 * rng.integers(0, max(1, (n - 1 - (c[-1] if L else 0)) // 8)))
-    ptr = np.zeros(m + 1, np.int64)
-    np.cumsum(lens, out=ptr[1:])
-    cols = np.concatenate(rows).astype(np.int32)
-    assert cols.max() < n
-    return m, n, ptr, cols, rng.uniform(-1, 1, ptr[-1])
+    if spacing is None:
+        cols = rng.integers(0, n, ptr[-1])
+        cols = cols[np.lexsort((cols, row))]
+    else:
+        step = e // 2 * spacing + e % 2 if kind.startswith("pairs") else e * spacing
+        room = n - 1 - (lens // 2 + 1) * spacing * (1 if kind.startswith("pairs") else 2)
+        cols = step + (8 * (rng.random(rows) * np.maximum(room, 8) // 8).astype(int))[row]
+    assert 0 <= cols.min() and cols.max() < n
+    return rows, n, ptr, cols.astype(np.int32), rng.uniform(-1, 1, ptr[-1])
 
 
 def spans(ptr, cols):
-    """Largest column span of a stored 64-entry block and of a stored 8-entry unit (full
-    blocks are stored transposed, 4 x 16)."""
-    block = unit = 0
-    for a, b in zip(ptr[:-1], ptr[1:]):
-        if a == b:
-            continue
-        c = np.concatenate([cols[a:b], np.full(-(b - a) % 8, cols[b - 1])]).astype(np.int64)
-        full = len(c) // 64 * 64
-        if full:
-            c[:full] = c[:full].reshape(-1, 4, 16).transpose(0, 2, 1).ravel()
-            block = max(block, int(np.ptp(c[:full].reshape(-1, 64), axis=1).max()))
-        if len(c) > full:
-            block = max(block, int(np.ptp(c[full:])))
-        unit = max(unit, int(np.ptp(c.reshape(-1, 8), axis=1).max()))
-    return block, unit
+    """Largest column span of a stored 64-entry block and of a stored 8-entry unit (rows
+    padded to 8 entries with their last column, full blocks stored transposed, 4 x 16)."""
+    lens = np.diff(ptr)
+    padded = (lens + 7) // 8 * 8
+    at = np.concatenate([[0], np.cumsum(padded)])
+    row = np.repeat(np.arange(len(lens)), padded)
+    q = np.arange(at[-1]) - at[row]
+    w = q % 64
+    e = np.where(q // 64 < padded[row] // 64, q - w + 16 * (w % 4) + w // 4, q)
+    stored = cols[ptr[row] + np.minimum(e, lens[row] - 1)].astype(np.int64)
+
+    def widest(starts):
+        return int((np.maximum.reduceat(stored, starts) - np.minimum.reduceat(stored, starts)).max())
+
+    return widest(np.flatnonzero(q % 64 == 0)), widest(np.flatnonzero(q % 8 == 0))
 
 
-CASES = [(kind, mean, fmt) for mean in (40, 80, 300) for kind, fmt in
-         (("pairs", "block"), ("pairs wide", "unit"), ("even", "block"), ("even wide", "unit"),
-          ("anywhere", "block"), ("anywhere wide", "none"))
-         # (a short row of a wide matrix fits in one block)
-         if not (mean == 40 and fmt == "unit")]
+CASES = [("pairs", 40, MANY, 0, "block"), ("anywhere", 40, MANY, 0, "block"),   # 32-bit columns
+         ("pairs", 40, MANY, 3000, "block"),                                    # a long row
+         ("pairs", 80, MANY, 0, "block"), ("pairs wide", 80, MANY, 0, "unit"),  # offsets
+         ("even", 110, MANY, 0, "block"), ("even wide", 110, MANY, 0, "unit"),  # scattered
+         ("anywhere", 110, MANY, 0, "block"),
+         ("pairs", 110, MANY, 0, "block"), ("pairs wide", 110, MANY, 0, "unit"),  # resident
+         ("pairs", 300, FEW, 0, "block"), ("even wide", 300, FEW, 0, "unit"),
+         ("anywhere", 300, FEW, 0, "block"),
+         ("anywhere wide", 110, MANY, 0, "none"), ("anywhere wide", 300, FEW, 0, "none")]
 
 
+@pytest.mark.parametrize("kind,mean,rows,longest,fmt", CASES)
 @pytest.mark.parametrize("vt", ["f32", "bf16"])
-@pytest.mark.parametrize("kind,mean,fmt", CASES)
-def test_products(vt, kind, mean, fmt):
+def test_products(vt, kind, mean, rows, longest, fmt):
     import torch
 
-    m, n, ptr, cols, vals = matrix(kind, mean)
+    m, n, ptr, cols, vals = matrix(kind, mean, rows, longest)
     assert ptr[-1] >= MIN_ENTRIES
     block, unit = spans(ptr, cols)
     assert (fmt == "block") == (block < 65536) and (fmt == "none") == (unit >= 65536)
@@ -100,20 +110,22 @@ def test_products(vt, kind, mean, fmt):
     stored = torch.from_numpy(vals).float()
     if vt == "bf16":
         stored = stored.bfloat16().float()
-    A = sp.csr_matrix((stored.double().numpy(), cols, ptr), shape=(m, n))
-    for M, v, y in ((A, x, u), (A.T.tocsr(), d, q)):
+    stored = stored.double().numpy()
+    # (scipy's abs() would add up a row's repeated columns first)
+    A, size = (sp.csr_matrix((a, cols, ptr), shape=(m, n)) for a in (stored, np.abs(stored)))
+    for M, S, v, y in ((A, size, x, u), (A.T.tocsr(), size.T.tocsr(), d, q)):
         v = v.astype(np.float64)
-        bound = (np.diff(M.indptr) + 2) * 2.0 ** -24 * (abs(M) @ np.abs(v))
+        bound = (np.diff(M.indptr) + 2) * 2.0 ** -24 * (S @ np.abs(v))
         assert np.all(np.abs(y - M @ v) <= bound)
 
 
 @pytest.mark.parametrize("nrhs", [3, 7, 16])
-@pytest.mark.parametrize("kind,mean", [("pairs", 300), ("pairs wide", 300), ("even wide", 80),
-                                       ("anywhere wide", 300)])
-def test_shared_products(kind, mean, nrhs):
+@pytest.mark.parametrize("kind,mean,rows", [("pairs", 300, FEW), ("pairs wide", 300, FEW),
+                                            ("even wide", 80, MANY), ("anywhere wide", 300, FEW)])
+def test_shared_products(kind, mean, rows, nrhs):
     """Four, eight and sixteen interleaved right-hand sides on large matrices: each solve has
     the bits of its own."""
-    m, n, ptr, cols, vals = matrix(kind, mean)
+    m, n, ptr, cols, vals = matrix(kind, mean, rows)
     K = 3
     b = np.random.default_rng(nrhs).standard_normal((nrhs, m))
     with lslu.BatchedSolver((m, n, ptr, cols, vals), "f32", K, nrhs=nrhs) as s:
